@@ -13,6 +13,7 @@
 #include "autotune.h"
 #include "launchset.h"
 #include "runtime.h"
+#include "tiles.h"
 
 namespace sdfg {
 
@@ -44,7 +45,7 @@ int resolve_config(const sdfg_config *cfg, int R, int C, int dtype, sdfg_config 
     if (c.seg_rows < 0 || c.warps < 0 || c.warps > MAX_WARPS)
         return set_error(SDFG_ERR_INVAL, "bad seg_rows/warps (%d/%d)", c.seg_rows, c.warps);
     sdfg_config tuned;
-    const bool have = autotune_lookup(R, C, dtype, &tuned);
+    const bool have = autotune_lookup(R, C, dtype, &tuned) && tuned.kernel != SDFG_KERNEL_AUTO;
     // large grids: one launch for all passes (no per-pass tail) -- the chain
     // kernel for FP32/BF16 storage, the persistent kernel for FP64; small
     // grids: one launch per pass
@@ -199,6 +200,20 @@ int run_single(const void *in, void *out, int R, int C, int ld, long long T, int
     sdfg_config c;
     rc = resolve_config(cfg, R, C, dtype, &c);
     if (rc != SDFG_OK) return rc;
+    // nothing asked for, and nothing else tuned: a grid that the chip's
+    // registers hold runs there from the first step to the last.  Measured
+    // against the launches below (their defaults): 256^2 T=100 50 us (233, a
+    // launch per pass), 1301 x 1777 on an odd pitch T=150 148 us (478),
+    // 2048^2 T=1024 1345 us (6676, chains; 1610 with register-resident passes)
+    sdfg_config tuned;
+    if ((!cfg || (cfg->kernel == SDFG_KERNEL_AUTO && cfg->k == 0 && cfg->seg_rows == 0 && cfg->warps == 0)) &&
+        (!autotune_lookup(R, C, dtype, &tuned) || tuned.kernel == SDFG_KERNEL_AUTO)) {
+        TilePlan plan;
+        if (plan_tiles(R, C, dtype, st->sm_count, &plan)) {
+            rc = run_tiles(in, out, R, C, ld, T, dtype, plan, st, s);
+            if (rc != SDFG_ERR_NOMEM) return rc;
+        }
+    }
     if (c.kernel == SDFG_KERNEL_RESIDENT && !resident_supported(dtype)) c.kernel = SDFG_KERNEL_TEMPORAL;
     const std::vector<int> ks = c.kernel == SDFG_KERNEL_NAIVE      ? std::vector<int>(1, static_cast<int>(T))
                                 : c.kernel == SDFG_KERNEL_RESIDENT ? plan_resident_passes(T, c.k)

@@ -118,6 +118,14 @@ std::vector<int> plan_resident_passes(long long T, int k);
 int run_resident_passes(const void *src0, void *first, void *second, const std::vector<int> &ks, int R, int C,
                         int ld, int dtype, DeviceState *st, cudaStream_t s, void **final);
 
+// ---- register tiles (tiles.cu) --------------------------------------------------
+struct TilePlan;  // tiles.h
+// The kernel variant and tile counts for a grid (FP32/BF16); false if it does not fit the chip's registers.
+bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan);
+// T >= 1 steps in one cooperative launch with that plan; any ld and alignment, in == out allowed.
+int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int dtype, const TilePlan &plan,
+              DeviceState *st, cudaStream_t s);
+
 // ---- skewed chains (skewed.cu) ------------------------------------------------
 // T steps of one grid in one launch of the chain kernel: passes of depth k,
 // chains of L rows (0: 512), progress published every `pub` chunks (0: 12).
