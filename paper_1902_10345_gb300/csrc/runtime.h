@@ -126,6 +126,9 @@ bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan);
 int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int dtype, const TilePlan &plan,
               DeviceState *st, cudaStream_t s);
 
+// The FP64 counterpart (tiles64.cu); *ran false: the grid does not fit, nothing was done.
+int run_tiles64(const void *in, void *out, int R, int C, int ld, long long T, DeviceState *st, cudaStream_t s, bool *ran);
+
 // ---- skewed chains (skewed.cu) ------------------------------------------------
 // T steps of one grid in one launch of the chain kernel: passes of depth k,
 // chains of L rows (0: 512), progress published every `pub` chunks (0: 12).
