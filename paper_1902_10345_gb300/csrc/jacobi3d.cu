@@ -4,11 +4,17 @@
 // interior point becomes
 //   (1/7) * (c + (((n + s) + (w + e)) + (u + d)))
 // (n, s: rows i-1, i+1; w, e: columns j-1, j+1; u, d: planes z-1, z+1), in
-// this order, round to nearest, no contraction, in the compute type (FP32 for
-// FP32 and BF16 storage, FP64 for FP64): an FP64 run equals the FP64
-// definition bit for bit.
+// this order, round to nearest, no contraction, in FP64 for FP64 storage (an
+// FP64 run equals the FP64 definition bit for bit) and in FP32 in the one-step
+// kernel below; the fused passes of FP32 and BF16 storage reassociate the sum
+// (jacobi3d_fused.cu).
 //
-// One launch is one timestep.  A CTA owns a tile of TY rows x TX columns and
+// Passes: FP32 and BF16 boxes advance 3 steps per launch, and 2 where T is no
+// multiple of 3 (jacobi3d_fused.cu; 512^3 T=100 17.5 -> 10.3 ms, a seventh of
+// the error); a single step runs on jacobi3d_kernel, FP64 on
+// jacobi3d_flat_kernel.
+//
+// jacobi3d_kernel: one launch is one timestep.  A CTA owns a tile of TY rows x TX columns and
 // streams through a range of planes (2.5-D blocking, paper App. B MapTiling
 // applied to rows and columns, the plane loop kept sequential): plane after
 // plane arrives by 3-D TMA -- the tile plus a one-row and a 16-byte column
@@ -22,6 +28,7 @@
 #include <algorithm>
 
 #include "device_common.cuh"
+#include "jacobi3d.h"
 #include "runtime.h"
 
 namespace sdfg {
@@ -340,10 +347,17 @@ extern "C" int sdfg_jacobi3d(const void *in, void *out, int depth, int rows, int
         return launch_copy2d(out, ld, in, ld, nr, cols, dtype, s);
     }
     const size_t S = dtype_bytes(dtype);
+    // FP32 and BF16 storage: passes of 3 fused steps, and of 2 where T is no
+    // multiple of 3; a single step runs alone
+    const bool f64 = dtype == SDFG_F64;
+    int n_two = 0, n_pass = T;
+    if (!f64 && T > 1) {
+        n_two = (3 - T % 3) % 3;
+        n_pass = n_two + (T - 2 * n_two) / 3;
+    }
     // ping-pong between two aligned boxes; unaligned or pitched-oddly
     // callers are staged through an aligned copy
     // (FP64 needs no alignment)
-    const bool f64 = dtype == SDFG_F64;
     const bool aligned = f64 || (j3_tma_ok(in, ld, dtype) && j3_tma_ok(out, ld, dtype));
     const int ldw = aligned ? ld : (cols + 31) / 32 * 32;
     const size_t bytes = static_cast<size_t>(n_rows) * ldw * S;
@@ -354,8 +368,8 @@ extern "C" int sdfg_jacobi3d(const void *in, void *out, int depth, int rows, int
         rc = scratch_alloc(&a, bytes, s);
         if (rc != SDFG_OK) return rc;
         if (in != out) {
-            // the last of T passes must land in `out`
-            first = (T % 2 == 1) ? out : a;
+            // the last pass must land in `out`
+            first = (n_pass % 2 == 1) ? out : a;
             second = first == out ? a : out;
         } else {
             first = a;
@@ -374,20 +388,43 @@ extern "C" int sdfg_jacobi3d(const void *in, void *out, int depth, int rows, int
         first = b;
         second = a;
     }
-    const int box_cols = j3_box_cols(dtype);
-    alignas(128) CUtensorMap tm_src0, tm_first, tm_second;
-    if (!f64) rc = encode_tmap3d(&tm_src0, src0, dtype, depth, rows, cols, ldw, box_cols, J3_BY);
-    if (!f64 && rc == SDFG_OK) rc = encode_tmap3d(&tm_first, first, dtype, depth, rows, cols, ldw, box_cols, J3_BY);
-    if (!f64 && rc == SDFG_OK) rc = encode_tmap3d(&tm_second, second, dtype, depth, rows, cols, ldw, box_cols, J3_BY);
-    const J3Geo g = plan_j3(depth, rows, cols, ldw, dtype, st->sm_count);
-    const CUtensorMap *tsrc = &tm_src0;
     void *dst = first;
     void *fin = const_cast<void *>(src0);
-    for (int t = 0; t < T && rc == SDFG_OK; ++t) {
-        rc = f64 ? launch_j3_flat(fin, dst, g, st->sm_count, s) : launch_j3(*tsrc, dst, g, dtype, st->d_err, s);
+    // the three buffers a pass may read: src0, first, second
+    alignas(128) CUtensorMap tm[3];
+    auto encode = [&](int box_cols, int box_rows) {
+        void *const bufs[3] = {const_cast<void *>(src0), first, second};
+        for (int i = 0; i < 3 && rc == SDFG_OK; ++i)
+            rc = encode_tmap3d(&tm[i], bufs[i], dtype, depth, rows, cols, ldw, box_cols, box_rows);
+    };
+    auto src_map = [&]() -> const CUtensorMap & { return fin == src0 ? tm[0] : fin == first ? tm[1] : tm[2]; };
+    auto done = [&]() {
         fin = dst;
-        tsrc = dst == first ? &tm_first : &tm_second;
         dst = dst == first ? second : first;
+    };
+    if (f64) {
+        const J3Geo g = plan_j3(depth, rows, cols, ldw, dtype, st->sm_count);
+        for (int t = 0; t < T && rc == SDFG_OK; ++t) {
+            rc = launch_j3_flat(fin, dst, g, st->sm_count, s);
+            done();
+        }
+    } else if (T == 1) {
+        encode(j3_box_cols(dtype), J3_BY);
+        if (rc == SDFG_OK) rc = launch_j3(tm[0], dst, plan_j3(depth, rows, cols, ldw, dtype, st->sm_count), dtype, st->d_err, s);
+        done();
+    } else {
+        // the fused kernel stores interior points only
+        rc = j3_shell_copy(src0, first, second == src0 || n_pass == 1 ? nullptr : second, depth, rows, cols, ldw, dtype, s);
+        for (int K : {3, 2}) {
+            const int n = K == 3 ? n_pass - n_two : n_two;
+            if (n == 0 || rc != SDFG_OK) continue;
+            encode(j3_fused_cols(), j3_fused_rows(K));
+            const J3FGeo g = j3_fused_plan(K, depth, rows, cols, ldw, dtype, st->sm_count);
+            for (int p = 0; p < n && rc == SDFG_OK; ++p) {
+                rc = launch_j3_fused(src_map(), dst, g, K, dtype, st->d_err, s);
+                done();
+            }
+        }
     }
     if (rc == SDFG_OK && fin != out) rc = launch_copy2d(out, ld, fin, ldw, nr, cols, dtype, s);
     scratch_free(a, s);
