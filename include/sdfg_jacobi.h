@@ -254,7 +254,8 @@ int sdfg_jacobi2d_batch(sdfg_desc *desc, int n, int check_stride, void *stream);
  * at the library's depth (8 for FP32/BF16, 4 for FP64) in one launch, every
  * other grid on the persistent kernel as above in a second launch; NULL: the
  * batch autotuner's cached choice for this class of batch, else the
- * persistent kernel.  Chains pay off for grids whose own work is long
+ * persistent kernel (with taller segments, and for FP32 depth 4, where a
+ * fixed-step batch has 12 M points or more).  Chains pay off for grids whose own work is long
  * (measured on 16 grids of 2048^2, 496 steps: 5064 against 3321 GUpdates/s);
  * on the uneven 512-grid batch the persistent kernel is faster.
  * plan_run is asynchronous; plan_results waits for the last run and fills

@@ -337,6 +337,25 @@ static void plan_free(sdfg_batch_plan *p) {
     delete p;
 }
 
+// Fused depth and segment height of an untuned fixed-step batch of `points`
+// points.  A small batch is bound by the lag from pass to pass: the defaults
+// (depth 8, 96 rows), deep passes of short units.  From about 12 M points on,
+// the warps in flight (12 per SM, 112 columns each) have several units a pass,
+// and throughput counts: units as tall as a third of the rows a warp has to
+// itself (halo rows), and for FP32 half the depth (fewer units that touch the
+// ring and fewer pipe variants in flight).  BF16 keeps the depth: its values
+// are rounded once a pass.  Measured, ms, defaults -> this: FP32, 512 grids of
+// 64..2048 (157 M points) 30.6 -> 15.4, 256 (83 M) 16.6 -> 9.6, 128 (44 M) 9.6
+// -> 6.2, 64 (22 M) 5.9 -> 3.8; below, depth 4 loses: 32 grids (8.8 M) 2.90 at
+// the defaults, 2.91; 128 grids of 64..512 (6.2 M) 2.8, 3.1.  BF16 157 M 32.7 ->
+// 27.1, 83 M 17.8 -> 16.6, 22 M 6.5 -> 6.3.
+static void untuned_batch(double points, int dtype, sdfg_config *c) {
+    if (dtype == SDFG_F64 || points < 12e6) return;
+    const int rows = static_cast<int>(points / (152 * 12 * 112) / 3) / 32 * 32;
+    c->seg_rows = std::min(256, std::max(dtype == SDFG_F32 ? 96 : 128, rows));
+    if (dtype == SDFG_F32) c->k = 4;
+}
+
 static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int check_stride, const sdfg_config *cfg,
                       bool use_graph) {
     *out = nullptr;
@@ -362,7 +381,10 @@ static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int c
         for (int g = 0; g < n; ++g) area += static_cast<double>(desc[g].rows) * desc[g].cols;
         area /= n;
         sdfg_config tuned;
-        if (autotune_lookup(-n, -static_cast<int>(area > 2e9 ? 2e9 : area), dtype, &tuned)) c = tuned;
+        if (autotune_lookup(-n, -static_cast<int>(area > 2e9 ? 2e9 : area), dtype, &tuned))
+            c = tuned;
+        else if (!any_tol)
+            untuned_batch(area * n, dtype, &c);
     }
     if (c.k != 0 && !depth_supported(c.k)) return set_error(SDFG_ERR_INVAL, "batch: k must be 1, 2, 4 or 8");
     if (c.warps < 0 || c.warps > MAX_WARPS || c.seg_rows < 0) return set_error(SDFG_ERR_INVAL, "batch: bad config");
