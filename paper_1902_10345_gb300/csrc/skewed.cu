@@ -291,15 +291,37 @@ int chain_plan_build(ChainPlan *c, DeviceState *st, cudaStream_t s) {
 }
 }  // namespace
 
+// Chain length and publication interval where the caller leaves them open.  A
+// pass trails the one before by the rows between two publications, and a chain
+// by its length: on a grid whose passes are short that lag sets the speed, and
+// short chains that publish every chunk win although each release stalls its
+// warp; on a large one the passes in flight hide it.  GUpdates/s at T=160,
+// 640-row chains publishing every 8 chunks -> this: FP32 2400^2 765 -> 1707,
+// 3000^2 1129 -> 2330, 4096^2 1979 -> 3599, 5600^2 3343 -> 4701, 7000^2 4614 ->
+// 5120, 8192^2 as before.  BF16 (512 rows, 6 chunks before) 2400^2 767 -> 1184,
+// 3000^2 1106 -> 1571, 4096^2 1817 -> 2319, 5600^2 2910 -> 3407, 7000^2 3727 ->
+// 4186; its warps hold two thirds more rows per chunk, so long chains that
+// publish every chunk beat short ones.
+static void chain_defaults(long long points, int dtype, int *L, int *pub) {
+    int l = 640, p = chain_pub_chunks(dtype_bytes(dtype));
+    if (dtype == SDFG_F32 && points < (58LL << 20)) {
+        l = 128;
+        p = points < (24LL << 20) ? 1 : points < (40LL << 20) ? 2 : 8;
+    } else if (dtype == SDFG_BF16) {
+        l = points < (8LL << 20) ? 256 : points < (58LL << 20) ? 640 : 512;
+        if (points < (58LL << 20)) p = 1;
+    }
+    if (*pub <= 0) *pub = *L <= 0 ? p : chain_pub_chunks(dtype_bytes(dtype));
+    if (*L <= 0) *L = l;
+}
+
 // The chain kernel's pass plan for T steps at depth k: plan_passes(T, k).
-// L: chain length in rows (0: 640, 512 for BF16 storage, the measured best);
-// pub: chunks between progress updates
-// (0 = about every 144 rows).  FP32, BF16 and FP64 storage; in/out must be
+// L: chain length in rows, pub: chunks between progress updates (0: see
+// chain_defaults; pub 0 with a given L: about every 144 rows).  FP32, BF16 and FP64 storage; in/out must be
 // TMA-compatible.
 int run_single_chain(const void *in, void *out, int R, int C, int ld, long long T, int dtype, int k, int L, int pub,
                      DeviceState *st, cudaStream_t s) {
-    if (L <= 0) L = dtype == SDFG_BF16 ? 512 : 640;
-    if (pub <= 0) pub = chain_pub_chunks(dtype_bytes(dtype));
+    chain_defaults(static_cast<long long>(R) * C, dtype, &L, &pub);
     L = std::max(L, 4 * k);
     std::lock_guard<std::mutex> lk(g_chain_mu);
     ChainPlan *c = nullptr;
