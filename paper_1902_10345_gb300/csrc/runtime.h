@@ -121,17 +121,18 @@ int run_resident_passes(const void *src0, void *first, void *second, const std::
 // ---- register tiles (tiles.cu) --------------------------------------------------
 struct TilePlan;  // tiles.h
 // The kernel variant and tile counts for a grid (FP32/BF16); false if it does not fit the chip's registers.
-bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan);
+bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan, bool sor = false);
 // T >= 1 steps in one cooperative launch with that plan; any ld and alignment, in == out allowed.
+// omega: T red-black SOR iterations instead (a plan made for them).
 int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int dtype, const TilePlan &plan,
-              DeviceState *st, cudaStream_t s);
+              DeviceState *st, cudaStream_t s, const double *omega = nullptr);
 
 // The FP64 counterpart (tiles64.cu); *ran false: the grid does not fit, nothing was done.
 int run_tiles64(const void *in, void *out, int R, int C, int ld, long long T, DeviceState *st, cudaStream_t s, bool *ran);
 
 // ---- skewed chains (skewed.cu) ------------------------------------------------
 // T steps of one grid in one launch of the chain kernel: passes of depth k,
-// chains of L rows (0: 512), progress published every `pub` chunks (0: 12).
+// chains of L rows, progress published every `pub` chunks (0: by the grid's size).
 // in/out must be TMA-compatible; in == out allowed.
 int run_single_chain(const void *in, void *out, int R, int C, int ld, long long T, int dtype, int k, int L, int pub,
                      DeviceState *st, cudaStream_t s);

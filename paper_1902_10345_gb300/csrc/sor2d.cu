@@ -22,6 +22,8 @@
 // sweeps.  Boundary-ring points are copied; every point of the grid is
 // written by exactly one CTA.
 //
+// Small FP32 and BF16 grids run on the register tiles instead (tiles.cuh).
+//
 // Two kernels.  FP64 storage (2 columns per lane) sweeps the box in shared
 // memory, on box rows [1 + h, BY - 1 - h) in half-sweep h.  FP32 and BF16
 // storage (4 columns per lane) load the box once into registers -- each warp
@@ -34,6 +36,8 @@
 
 #include "device_common.cuh"
 #include "runtime.h"
+#include "sor_row.cuh"
+#include "tiles.h"
 
 namespace sdfg {
 
@@ -235,49 +239,6 @@ template <int I, int N, class F> __device__ __forceinline__ void static_for(F &&
         f(std::integral_constant<int, I>());
         static_for<I + 1, N>(f);
     }
-}
-
-// Packed FP32x2 add, rounded to nearest.
-__device__ __forceinline__ float2 add2_rn(float2 x, float2 y) {
-    float2 r;
-    asm("{\n\t.reg .b64 a, b, d;\n\t"
-        "mov.b64 a, {%2, %3};\n\t"
-        "mov.b64 b, {%4, %5};\n\t"
-        "add.rn.f32x2 d, a, b;\n\t"
-        "mov.b64 {%0, %1}, d;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y));
-    return r;
-}
-// One row of a half-sweep in registers.  Lane l holds the row's columns
-// 4l .. 4l+3 in c; a row of colour parity P updates its elements P and P+2
-// in place from the rows above (n) and below (s) -- of which only elements P
-// and P+2 are read: they have the other colour -- and from c's other two
-// elements.  The same operations, in the same order, as sor_point, each
-// rounded on its own: the sums two points per packed FP32x2 add, the products
-// scalar.  BF16 storage rounds the new values to BF16.
-template <bool BF, int P, bool EDGE>
-__device__ __forceinline__ void sor_row_reg(const float (&n)[4], float (&c)[4], const float (&s)[4], float a,
-                                            float b, bool row_in, unsigned colin) {
-    float2 we;
-    if constexpr (P == 0) {
-        const float left = __shfl_up_sync(FULL_MASK, c[3], 1);
-        we = make_float2(__fadd_rn(left, c[1]), __fadd_rn(c[1], c[3]));
-    } else {
-        const float right = __shfl_down_sync(FULL_MASK, c[0], 1);
-        we = make_float2(__fadd_rn(c[0], c[2]), __fadd_rn(c[2], right));
-    }
-    const float2 ns = add2_rn(make_float2(n[P], n[P + 2]), make_float2(s[P], s[P + 2]));
-    const float2 q = add2_rn(ns, we);
-    // the products are scalar: the code generator may fuse a packed product
-    // that has a single use into the packed add consuming it (one rounding
-    // instead of two), even when both carry an explicit rounding mode
-    const float2 ac = make_float2(__fmul_rn(a, c[P]), __fmul_rn(a, c[P + 2]));
-    const float2 bq = make_float2(__fmul_rn(b, q.x), __fmul_rn(b, q.y));
-    float2 v = add2_rn(ac, bq);
-    if constexpr (BF) v = __bfloat1622float2(__float22bfloat162_rn(v));
-    if (!EDGE || (row_in && ((colin >> P) & 1u))) c[P] = v.x;
-    if (!EDGE || (row_in && ((colin >> (P + 2)) & 1u))) c[P + 2] = v.y;
 }
 
 // Warp w holds box rows [w RB, w RB + RB) in registers.  Between half-sweeps
@@ -505,6 +466,20 @@ extern "C" int sdfg_sor2d(const void *in, void *out, int rows, int cols, int ld,
     if (T == 0 || rows < 3 || cols < 3) {
         if (in == out) return SDFG_OK;
         return launch_copy2d(out, ld, in, ld, rows, cols, dtype, s);
+    }
+    // A small grid runs in one launch, held in registers (tiles.cuh), any layout:
+    // a pass of 4 iterations takes 3.3 us there at the least, the launches below
+    // 6.3, and more points per SM bring them together at about 2.4 M; the
+    // cooperative launch costs about 8 us more than a plain one, so few
+    // iterations stay below.  us at T=100, launches -> tiles: 256^2 158 -> 89,
+    // 500^2 158 -> 104, 777 x 1023 (odd pitch) 170 -> 133, 1000^2 159 -> 134,
+    // 1500^2 261 -> 230, 1800^2 311 -> 355; T=8: 1000^2 18 -> 23.
+    if (dtype != SDFG_F64 && T >= 32 && static_cast<long long>(rows) * cols <= 2400000) {
+        TilePlan plan;
+        if (plan_tiles(rows, cols, dtype, st->sm_count, &plan, true)) {
+            rc = run_tiles(in, out, rows, cols, ld, T, dtype, plan, st, s, &omega);
+            if (rc != SDFG_ERR_NOMEM) return rc;
+        }
     }
     const size_t S = dtype_bytes(dtype);
     int ki, box_cols, tile_cols, box_rows, tile_rows;

@@ -12,13 +12,17 @@ namespace sdfg {
 const void *tile_fn_mid(int rb, int dtype);   // tiles_mid.cu: 16 warps, up to 9 rows
 const void *tile_fn_tall(int rb, int dtype);  // tiles_tall.cu: up to 12
 const void *tile_fn_top(int rb, int dtype);   // tiles_top.cu: up to 18
+const void *sor_tile_fn(TileShape v, int dtype);       // sor_tiles.cu
+const void *sor_tile_fn_tall(TileShape v, int dtype);  // sor_tiles_tall.cu: 16 warps, 10 rows and more
 
 namespace {
 constexpr TileShape kShapes[] = {{8, 4},   {8, 5},   {8, 6},   {8, 7},   {16, 4},  {16, 5},  {16, 6},  {16, 7}, {16, 8},
                                  {16, 9},  {16, 10}, {16, 11}, {16, 12}, {16, 14}, {16, 16}, {16, 17}, {16, 18}};
 constexpr int kShapeCount = sizeof(kShapes) / sizeof(kShapes[0]);
+bool sor_has(TileShape v) { return v.nw == 8 ? v.rb % 2 == 0 : v.rb % 2 == 0 ? v.rb < 16 : v.rb == 17; }
 
-const void *tile_fn(TileShape v, int dtype) {
+const void *tile_fn(TileShape v, int dtype, bool sor) {
+    if (sor) return v.nw == 16 && v.rb >= 10 ? sor_tile_fn_tall(v, dtype) : sor_tile_fn(v, dtype);
     if (v.nw == 16) return v.rb <= 9 ? tile_fn_mid(v.rb, dtype) : v.rb <= 12 ? tile_fn_tall(v.rb, dtype) : tile_fn_top(v.rb, dtype);
     switch (v.rb) {
         case 4: return tile_fn_of<8, 4>(dtype);
@@ -29,14 +33,14 @@ const void *tile_fn(TileShape v, int dtype) {
 }
 
 // CTAs of variant `i` an SM holds (a property of the compiled kernel)
-int tile_blocks_per_sm(int i, int dtype) {
+int tile_blocks_per_sm(int i, int dtype, bool sor) {
     static std::mutex mu;
-    static int cache[kShapeCount][2];
+    static int cache[kShapeCount][2][2];
     std::lock_guard<std::mutex> lk(mu);
-    int &n = cache[i][dtype == SDFG_BF16];
+    int &n = cache[i][dtype == SDFG_BF16][sor];
     if (n == 0) {
         const TileShape v = kShapes[i];
-        const void *fn = tile_fn(v, dtype);
+        const void *fn = tile_fn(v, dtype, sor);
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(tile_smem(v))) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, 32 * v.nw, tile_smem(v)) != cudaSuccess) {
             cudaGetLastError();
@@ -70,7 +74,7 @@ template <class First> bool halos_in_neighbours(int n, int extent, int tile, int
 // neighbouring band's row.  Measured best and chosen: 256^2 T=100 8 warps x 4
 // rows (50 us; 7 rows 54, 16 x 4 60), 1301 x 1777 T=150 16 x 12 (146 us) and
 // 16 x 11 (148), 2048^2 T=1024 16 x 17 (1345 us; 16 x 18 1450).
-bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan) {
+bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan, bool sor) {
     if (dtype == SDFG_F64 || R < 3 || C < 3) return false;
     const int x = tiles_along(C, TK_TX);
     if (x > 4LL * sm_count) return false;
@@ -78,13 +82,14 @@ bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan) {
     double best = 0.0;
     for (int i = 0; i < kShapeCount; ++i) {
         const TileShape v = kShapes[i];
+        if (sor && !sor_has(v)) continue;
         const int TY = tile_rows(v);
         if (R < TY) continue;  // the ring rows lie at fixed box rows: a tile is no taller than the grid
         const int y = tiles_along(R, TY);
         const long long n = static_cast<long long>(x) * y;
         if (n > 4LL * sm_count || !halos_in_neighbours(y, R, TY, TK_HALO, [&](int t) { return tile_y0_of(R, y, t, TY); }))
             continue;
-        if (n > static_cast<long long>(tile_blocks_per_sm(i, dtype)) * sm_count) continue;
+        if (n > static_cast<long long>(tile_blocks_per_sm(i, dtype, sor)) * sm_count) continue;
         const int per_sm = static_cast<int>((n + sm_count - 1) / sm_count);
         const double cost = 8.0 * (14.0 * v.rb * (v.nw / 4) * per_sm + 250.0);
         if (best == 0.0 || cost < best) {
@@ -98,7 +103,7 @@ bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan) {
 }
 
 int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int dtype, const TilePlan &plan,
-              DeviceState *st, cudaStream_t s) {
+              DeviceState *st, cudaStream_t s, const double *omega) {
     const int nx = plan.nx, ny = plan.ny;
     TileParams p;
     memset(&p, 0, sizeof(p));
@@ -113,8 +118,13 @@ int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int 
     p.ny = ny;
     const size_t quad = 4 * static_cast<size_t>(dtype_bytes(dtype));
     p.vec = reinterpret_cast<uintptr_t>(in) % quad == 0 && reinterpret_cast<uintptr_t>(out) % quad == 0 && ld % 4 == 0;
-    p.n_pass = static_cast<int>((T + TK_HALO - 1) / TK_HALO);
-    p.k_last = static_cast<int>(T - static_cast<long long>(p.n_pass - 1) * TK_HALO);
+    const int per_step = omega ? 2 : 1;  // an SOR iteration is two half-sweeps, each a cell of halo
+    p.n_pass = static_cast<int>((T * per_step + TK_HALO - 1) / TK_HALO);
+    p.k_last = static_cast<int>(T * per_step - static_cast<long long>(p.n_pass - 1) * TK_HALO);
+    if (omega) {
+        p.a = static_cast<float>(1.0 - *omega);
+        p.b = static_cast<float>(0.25 * *omega);
+    }
     auto split = [](int k, float *hi, float *lo) {
         double f = 1.0;
         for (int i = 0; i < k; ++i) f = 0.2 * f;
@@ -139,8 +149,8 @@ int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int 
     cudaError_t e = words ? cudaMemsetAsync(ws, 0, words, s) : cudaSuccess;
     if (e == cudaSuccess) {
         void *args[] = {&p};
-        TimedLaunch t = stats_begin(FAM_RESIDENT, s);
-        e = cudaLaunchCooperativeKernel(tile_fn(plan.shape, dtype), dim3(nx * ny), dim3(32 * plan.shape.nw), args,
+        TimedLaunch t = stats_begin(omega ? FAM_SOR : FAM_RESIDENT, s);
+        e = cudaLaunchCooperativeKernel(tile_fn(plan.shape, dtype, omega != nullptr), dim3(nx * ny), dim3(32 * plan.shape.nw), args,
                                         tile_smem(plan.shape), s);
         stats_end(t, s);
     }

@@ -28,7 +28,10 @@
 // pass, so two CTAs of an SM compute at the same time and wait at the same
 // time (12.4 us per pass with 304 tiles of 8 x 18, 10.9 with 152).
 //
-// Arithmetic: (n + (w + c + e)) + s with shared pair sums, unscaled (after t
+// The same kernel runs red-black SOR (SOR: 8 half-sweeps, 4 iterations, per
+// pass, in the exact order of sor2d.cu).
+//
+// Arithmetic (Jacobi): (n + (w + c + e)) + s with shared pair sums, unscaled (after t
 // steps of a pass the tile holds 5^t times the state), one multiplication by
 // 0.2^8 (hi + lo) at the end of a pass.  The order does not depend on a
 // point's place in its tile, so the tiling changes no bit.  The boundary ring
@@ -41,6 +44,7 @@
 #include <type_traits>
 
 #include "exchange.cuh"
+#include "sor_row.cuh"
 #include "tiles.h"
 
 namespace sdfg {
@@ -106,7 +110,7 @@ struct TilePlace {
     }
 };
 
-template <class ST, int NW, int RB>
+template <class ST, int NW, int RB, bool SOR>
 __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_constant__ TileParams P) {
     constexpr int NT = 32 * NW;
     constexpr int BY = NW * RB;
@@ -273,28 +277,75 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
         put(bot[slot ^ 1][warp + 1], o);
     };
 
+    // One red-black half-sweep (SOR): the rows' points of one colour, in place;
+    // a point reads only points of the other colour, which do not change.  PAR:
+    // the parity of the band's first row; EDGE: the box may hold points that
+    // keep their values.
+    auto half_sweep = [&](auto par_t, auto edge_t, int slot, int yb, unsigned colin) {
+        constexpr int PAR = decltype(par_t)::value;
+        constexpr bool EDGE = decltype(edge_t)::value;
+        constexpr bool BF = sizeof(ST) == 2;
+        auto row = [&](auto i_t, const float(&n)[4], const float(&s)[4]) {
+            constexpr int i = decltype(i_t)::value;
+            sor_row_reg<BF, PAR ^ (i & 1), EDGE>(n, X[i], s, P.a, P.b, !EDGE || (yb + i >= 1 && yb + i <= R - 2), colin);
+        };
+        tk_for<1, RB - 1>([&](auto i_t) { row(i_t, X[decltype(i_t)::value - 1], X[decltype(i_t)::value + 1]); });
+        __syncthreads();
+        float nb[4];
+        get(nb, bot[slot][warp]);
+        row(std::integral_constant<int, 0>(), nb, X[1]);
+        put(top[slot ^ 1][warp], X[0]);
+        get(nb, top[slot][warp + 1]);
+        row(std::integral_constant<int, RB - 1>(), X[RB - 2], nb);
+        put(bot[slot ^ 1][warp + 1], X[RB - 1]);
+    };
+
     LLWait wait{P.timeout_ns, P.err, false};
     for (int pass = 0; pass < P.n_pass; ++pass) {
         const bool last = pass == P.n_pass - 1;
         const int nk = last ? P.k_last : TK_HALO;
         put(top[0][warp], X[0]);
         put(bot[0][warp + 1], X[RB - 1]);
-        auto steps = [&](auto cf_t) {
+        if constexpr (SOR) {
+            const TilePlace g = *where();
+            const int yb = g.y0 - TK_HALO + warp * RB, gx = g.x0 - TK_HALO + lane * 4;
+            const bool edge = variant || g.ty == 0 || g.ty == P.ny - 1;
+            unsigned colin = 0;  // interior columns among the lane's four
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (gx + e >= 1 && gx + e <= C - 2) colin |= 1u << e;
+            using Even = std::integral_constant<int, 0>;
+            using Odd = std::integral_constant<int, 1>;
+            using Edge = std::true_type;
+            using Plain = std::false_type;
+            // red (even row + column) first; x0 is even, and so is each lane's column
 #pragma unroll 1
-            for (int t = 0; t < nk; ++t) step(cf_t, t & 1);
-        };
-        switch (variant) {
-            case 0: steps(std::integral_constant<int, 0>()); break;
-            case 1: steps(std::integral_constant<int, 1>()); break;
-            case 2: steps(std::integral_constant<int, 2>()); break;
-            case 3: steps(std::integral_constant<int, 3>()); break;
-            case 4: steps(std::integral_constant<int, 4>()); break;
-            case 5: steps(std::integral_constant<int, 5>()); break;
-            default: steps(std::integral_constant<int, 6>()); break;
+            for (int t = 0; t < nk; ++t) {
+                if ((yb + t) & 1)
+                    edge ? half_sweep(Odd(), Edge(), t & 1, yb, colin) : half_sweep(Odd(), Plain(), t & 1, yb, colin);
+                else
+                    edge ? half_sweep(Even(), Edge(), t & 1, yb, colin) : half_sweep(Even(), Plain(), t & 1, yb, colin);
+            }
+        } else {
+            auto steps = [&](auto cf_t) {
+#pragma unroll 1
+                for (int t = 0; t < nk; ++t) step(cf_t, t & 1);
+            };
+            switch (variant) {
+                case 0: steps(std::integral_constant<int, 0>()); break;
+                case 1: steps(std::integral_constant<int, 1>()); break;
+                case 2: steps(std::integral_constant<int, 2>()); break;
+                case 3: steps(std::integral_constant<int, 3>()); break;
+                case 4: steps(std::integral_constant<int, 4>()); break;
+                case 5: steps(std::integral_constant<int, 5>()); break;
+                default: steps(std::integral_constant<int, 6>()); break;
+            }
         }
-        // the box to shared memory, times 0.2^nk as hi + lo (the product is
-        // rounded once from a ~48-bit factor)
-        {
+        // the box to shared memory, for Jacobi times 0.2^nk as hi + lo (the
+        // product is rounded once from a ~48-bit factor)
+        if constexpr (SOR) {
+            tk_for<0, RB>([&](auto i_t) { put(band + decltype(i_t)::value * 32, X[decltype(i_t)::value]); });
+        } else {
             const float hi = last ? P.hi_last : P.hi, lo = last ? P.lo_last : P.lo;
             const float2 h2 = make_float2(hi, hi), l2 = make_float2(lo, lo);
             tk_for<0, RB>([&](auto i_t) {
@@ -307,8 +358,8 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
         __syncthreads();
         const TilePlace g = *where();
         const int tx = g.tx, ty = g.ty;
-        // the ring's exact values
-        if (variant || ty == 0 || ty == P.ny - 1) {
+        // the ring's exact values (SOR never changes them)
+        if (!SOR && (variant || ty == 0 || ty == P.ny - 1)) {
             if (tid < BY && tx == 0) box[tid][TK_HALO] = ring_col[0][tid];
             if (tid < BY && tx == P.nx - 1) box[tid][rq] = ring_col[1][tid];
             if (tid < TK_W && ty == 0) box[TK_HALO][tid] = ring_row[0][tid];
@@ -425,9 +476,9 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
     }
 }
 
-template <int NW, int RB> const void *tile_fn_of(int dtype) {
-    return dtype == SDFG_BF16 ? reinterpret_cast<const void *>(&tile_kernel<__nv_bfloat16, NW, RB>)
-                              : reinterpret_cast<const void *>(&tile_kernel<float, NW, RB>);
+template <int NW, int RB, bool SOR = false> const void *tile_fn_of(int dtype) {
+    return dtype == SDFG_BF16 ? reinterpret_cast<const void *>(&tile_kernel<__nv_bfloat16, NW, RB, SOR>)
+                              : reinterpret_cast<const void *>(&tile_kernel<float, NW, RB, SOR>);
 }
 
 }  // namespace sdfg

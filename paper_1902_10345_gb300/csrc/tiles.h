@@ -20,8 +20,9 @@ struct TileParams {
     int R, C, ld, ldx;
     int nx, ny;       // tiles
     int vec;          // rows can be read and written four columns at a time
-    int n_pass, k_last;  // passes, steps of the last one
+    int n_pass, k_last;  // passes, steps (SOR: half-sweeps) of the last one
     float hi, lo, hi_last, lo_last;  // 0.2^8 and 0.2^k_last as hi + lo
+    float a, b;       // SOR: 1 - omega, omega / 4
     unsigned long long timeout_ns;
 };
 
