@@ -28,13 +28,15 @@
  *     carry the unscaled 5-point sums through the k fused steps of a pass and
  *     multiply by 0.2^k once, at the pass's last step -- which saves about a
  *     quarter of the FP32 work and is more accurate against FP64, not less.
+ *     The chain kernel and the register tiles reassociate everywhere, and so
+ *     do the fused passes of the 3-D stencil (sums scaled by 7^-k).
  *     FP32 results are therefore bit-identical for the same geometry (fused
  *     depth k and segment height, hence alone or in any batch or server mix),
  *     and agree with other geometries to within the FP32 tolerance (max-abs
  *     1e-4 on fields in [0, 1]) rather than bit for bit.
  *   - BF16 storage: the steps fused into one pass stay in FP32 registers and
  *     values are rounded to BF16 each time a pass writes the grid, so the
- *     result also depends on k.
+ *     result also depends on k; the register tiles round once, at the end.
  *
  * Storage types: FP32 (arithmetic FP32), BF16 (the grid is stored in BF16;
  * arithmetic is FP32, and the steps fused into one pass stay in FP32
@@ -89,7 +91,12 @@ typedef enum {
 
 /* Kernel families for sdfg_config.kernel. */
 typedef enum {
-    SDFG_KERNEL_AUTO = 0,       /* autotuned choice                          */
+    SDFG_KERNEL_AUTO = 0,       /* autotuned choice; untuned, with every other
+                                   field 0: a grid that the SMs' registers
+                                   (FP64: shared memory) hold in one
+                                   cooperative launch of all steps, larger
+                                   ones on the chain kernel (FP64: one step
+                                   per launch)                              */
     SDFG_KERNEL_NAIVE = 1,      /* one timestep per launch, one thread/point */
     SDFG_KERNEL_TEMPORAL = 2,   /* k timesteps per launch (one pass)         */
     SDFG_KERNEL_PERSISTENT = 3, /* one launch for all passes, dependency-driven */
@@ -99,8 +106,8 @@ typedef enum {
                                    for grids that fit in L2, where a pass is
                                    latency-bound                            */
     SDFG_KERNEL_SKEWED = 5      /* one launch for all passes; each warp streams
-                                   a chain of seg_rows rows (0: 640, 512 for
-                                   BF16 storage) of one
+                                   a chain of seg_rows rows (0: by the grid's
+                                   size, 128 to 640) of one
                                    column strip through the k fused steps,
                                    chains skewed down by k rows per pass so
                                    that no rows are recomputed between them;
@@ -254,8 +261,9 @@ int sdfg_jacobi2d_batch(sdfg_desc *desc, int n, int check_stride, void *stream);
  * at the library's depth (8 for FP32/BF16, 4 for FP64) in one launch, every
  * other grid on the persistent kernel as above in a second launch; NULL: the
  * batch autotuner's cached choice for this class of batch, else the
- * persistent kernel (with taller segments, and for FP32 depth 4, where a
- * fixed-step batch has 12 M points or more).  Chains pay off for grids whose own work is long
+ * persistent kernel (a fixed-step FP32 or BF16 batch of 2^18 points or more
+ * with depth and segment height by its size and every unit reassociated).
+ * Chains pay off for grids whose own work is long
  * (measured on 16 grids of 2048^2, 496 steps: 5064 against 3321 GUpdates/s);
  * on the uneven 512-grid batch the persistent kernel is faster.
  * plan_run is asynchronous; plan_results waits for the last run and fills
@@ -315,9 +323,11 @@ int sdfg_laplace1d(double *A, int N, int T, void *stream);
  * timesteps every interior point becomes
  *   (1/7) * (c + (((n + s) + (w + e)) + (u + d)))
  * (n, s: rows i-1, i+1; w, e: columns j-1, j+1; u, d: planes z-1, z+1), in
- * that order, round to nearest, in FP32 (FP32 and BF16 storage; BF16 is
- * rounded when each step is stored) or FP64 (bit-identical to a plain FP64
- * loop).  The one-cell outer shell keeps its input values.  out receives the
+ * that order, round to nearest, in FP64 for FP64 (bit-identical to a plain FP64
+ * loop).  FP32 and BF16 storage compute in FP32 and, from T = 2 on, fuse two or
+ * three steps per pass: sums carried unscaled in another order and scaled once
+ * per pass, which is more accurate against FP64; BF16 is rounded when a pass
+ * stores the box.  The one-cell outer shell keeps its input values.  out receives the
  * whole box after T steps; in is read only; in == out is allowed; T = 0, or
  * an extent below 3, copies.  in/out should be 16-byte aligned with ld *
  * sizeof(element) a multiple of 16; otherwise the box is staged through an

@@ -223,7 +223,7 @@ int LaunchSet::upload(cudaStream_t s) {
     DeviceState *st = nullptr;
     int rc = current_device(&st);
     if (rc != SDFG_OK) return rc;
-    const int bps = std::max(1, persistent_blocks_per_sm(dtype, warps));
+    const int bps = std::max(1, persistent_blocks_per_sm(dtype, warps, scaled_edges));
     const long long need = (static_cast<long long>(total_items) + warps - 1) / warps;
     blocks = static_cast<int>(std::max<long long>(1, std::min<long long>(need, static_cast<long long>(bps) * st->sm_count)));
     return SDFG_OK;
@@ -249,7 +249,7 @@ int enqueue_persistent(LaunchSet &ls, DeviceState *st, cudaStream_t s) {
     int rc = ls.reset(s);
     if (rc != SDFG_OK) return rc;
     ls.L.err = st->d_err;
-    return launch_persistent(ls.L, ls.dtype, ls.warps, ls.blocks, s);
+    return launch_persistent(ls.L, ls.dtype, ls.warps, ls.blocks, ls.scaled_edges, s);
 }
 
 }  // namespace sdfg
@@ -272,6 +272,8 @@ struct sdfg_batch_plan {
     ChainBatch cb;           // large fixed-step grids on the skewed-chain kernel
     std::vector<char> on_chain;
     int n_pers = 0, n_chain = 0;
+    void *d_ring = nullptr;   // ring copies of the persistent grids (scaled edges)
+    int n_ring = 0, max_ring = 0;
     void *d_final = nullptr;  // finalise descriptors of the persistent grids
     int n_final = 0;
     int max_rows = 0;
@@ -310,7 +312,9 @@ static int plan_enqueue(sdfg_batch_plan *p, cudaStream_t s) {
         if (rc != SDFG_OK) return rc;
     }
     if (p->n_pers) {
-        rc = enqueue_persistent(p->ls, p->st, s);
+        if (p->n_ring)
+            rc = launch_ring_copy(static_cast<const RingCopy *>(p->d_ring), p->n_ring, p->max_ring, p->dtype, s);
+        if (rc == SDFG_OK) rc = enqueue_persistent(p->ls, p->st, s);
         if (rc != SDFG_OK) return rc;
         if (p->n_final)
             rc = launch_finalize(p->d_final, p->n_final, p->ls.L.grids, p->ls.L.state, p->dtype, p->max_rows, s);
@@ -325,6 +329,7 @@ static void plan_free(sdfg_batch_plan *p) {
     if (p->exec) cudaGraphExecDestroy(p->exec);
     if (p->graph) cudaGraphDestroy(p->graph);
     for (void *b : p->owned) cudaFreeAsync(b, s);
+    if (p->d_ring) cudaFreeAsync(p->d_ring, s);
     if (p->d_final) cudaFreeAsync(p->d_final, s);
     if (p->d_gcopy) cudaFreeAsync(p->d_gcopy, s);
     p->ls.release(s);
@@ -337,23 +342,38 @@ static void plan_free(sdfg_batch_plan *p) {
     delete p;
 }
 
-// Fused depth and segment height of an untuned fixed-step batch of `points`
-// points.  A small batch is bound by the lag from pass to pass: the defaults
-// (depth 8, 96 rows), deep passes of short units.  From about 12 M points on,
-// the warps in flight (12 per SM, 112 columns each) have several units a pass,
-// and throughput counts: units as tall as a third of the rows a warp has to
-// itself (halo rows), and for FP32 half the depth (fewer units that touch the
-// ring and fewer pipe variants in flight).  BF16 keeps the depth: its values
-// are rounded once a pass.  Measured, ms, defaults -> this: FP32, 512 grids of
-// 64..2048 (157 M points) 30.6 -> 15.4, 256 (83 M) 16.6 -> 9.6, 128 (44 M) 9.6
-// -> 6.2, 64 (22 M) 5.9 -> 3.8; below, depth 4 loses: 32 grids (8.8 M) 2.90 at
-// the defaults, 2.91; 128 grids of 64..512 (6.2 M) 2.8, 3.1.  BF16 157 M 32.7 ->
-// 27.1, 83 M 17.8 -> 16.6, 22 M 6.5 -> 6.3.
-static void untuned_batch(double points, int dtype, sdfg_config *c) {
-    if (dtype == SDFG_F64 || points < 12e6) return;
+// How an untuned fixed-step batch of n grids and `points` points runs: fused
+// depth, segment height, and (the result) whether every unit takes the
+// reassociated pipe, the ring held scaled -- an eighth of the error against FP64
+// of exact-order boundary units, and fewer pipe variants in flight.
+// - Below 2^18 points, FP64, and for BF16 between 3 M and 12 M points and for
+//   large batches of small grids: as a batch with tolerance grids, depth 8, 96
+//   rows, exact order at the ring.
+// - Below 12 M points the lag from pass to pass counts: depth 8, 64 rows.
+// - From there on the warps in flight (12 per SM, 112 columns each) have several
+//   units a pass: units as tall as a third of the rows a warp has to itself
+//   (fewer halo rows), FP32 at depth 4 (which loses 2 to 7% to depth 8 on some
+//   batches and wins 20% on 384 grids of 64..512); BF16 keeps the depth, as its
+//   values are rounded once a pass.
+// Measured, ms, before -> now (points; grids of 64..2048 if not said): FP32 512
+// grids (157 M) 30.6 -> 15.1, 256 (83 M) 16.6 -> 8.9, 128 (44 M) 9.6 -> 5.6, 64
+// (22 M) 5.9 -> 3.5, 384 of 64..512 (18 M) 5.7 -> 3.8, 32 (9 M) 2.9 -> 1.9, 16
+// (2 M) 2.0 -> 1.45, 12 of 64..300 (0.3 M) 1.5 -> 1.2; BF16 157 M 32.7 -> 23.8,
+// 44 M 10.4 -> 8.8, 2 M 2.1 -> 1.5, but 384 of 64..512 6.3 -> 6.8, 128 of them
+// (6 M) 3.1 -> 3.4, so those stay.
+static bool untuned_batch(double points, int n, int dtype, sdfg_config *c) {
+    const bool bf16 = dtype == SDFG_BF16;
+    if (dtype == SDFG_F64 || points < (1 << 18)) return false;
+    if (points < 12e6) {
+        if (bf16 && points >= 3e6) return false;
+        c->seg_rows = 64;
+        return true;
+    }
+    if (bf16 && points / n < (1 << 17)) return false;
     const int rows = static_cast<int>(points / (152 * 12 * 112) / 3) / 32 * 32;
-    c->seg_rows = std::min(256, std::max(dtype == SDFG_F32 ? 96 : 128, rows));
-    if (dtype == SDFG_F32) c->k = 4;
+    c->seg_rows = std::min(256, std::max(bf16 ? 128 : 96, rows));
+    if (!bf16) c->k = 4;
+    return true;
 }
 
 static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int check_stride, const sdfg_config *cfg,
@@ -374,6 +394,7 @@ static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int c
     }
     if (any_tol && check_stride < 1) return set_error(SDFG_ERR_INVAL, "batch: check_stride must be >= 1");
     sdfg_config c = {SDFG_KERNEL_PERSISTENT, 0, 0, 0};
+    bool scaled_edges = false;
     if (cfg) {
         c = *cfg;
     } else if (n > 0) {
@@ -384,7 +405,7 @@ static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int c
         if (autotune_lookup(-n, -static_cast<int>(area > 2e9 ? 2e9 : area), dtype, &tuned))
             c = tuned;
         else if (!any_tol)
-            untuned_batch(area * n, dtype, &c);
+            scaled_edges = untuned_batch(area * n, n, dtype, &c);
     }
     if (c.k != 0 && !depth_supported(c.k)) return set_error(SDFG_ERR_INVAL, "batch: k must be 1, 2, 4 or 8");
     if (c.warps < 0 || c.warps > MAX_WARPS || c.seg_rows < 0) return set_error(SDFG_ERR_INVAL, "batch: bad config");
@@ -404,6 +425,7 @@ static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int c
     p->ls.k = c.k ? c.k : default_depth(dtype);
     p->ls.warps = c.warps ? c.warps : 4;
     p->ls.check_stride = p->check_stride;
+    p->ls.scaled_edges = scaled_edges;
     cudaError_t e = cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->done_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
@@ -510,6 +532,28 @@ static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int c
         }
     }
     if (rc == SDFG_OK) rc = p->ls.build(runs_p);
+    if (rc == SDFG_OK && p->ls.scaled_edges) {
+        std::vector<RingCopy> rings;
+        for (const GridRun &r : runs_p) {
+            RingCopy q{};
+            q.src = r.buf[r.cur];
+            int nd = 0;
+            for (int i = 0; i < 2; ++i)
+                if (r.buf[i] && r.buf[i] != q.src) q.dst[nd++] = r.buf[i];
+            q.R = r.R;
+            q.C = r.C;
+            q.ld = r.ld;
+            rings.push_back(q);
+            p->max_ring = std::max(p->max_ring, 2 * r.C + 2 * (r.R - 2));
+        }
+        rc = scratch_alloc(&p->d_ring, rings.size() * sizeof(RingCopy), s);
+        if (rc == SDFG_OK && !rings.empty()) {
+            e = cudaMemcpyAsync(p->d_ring, rings.data(), rings.size() * sizeof(RingCopy), cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) rc = cuda_error(e, "batch plan upload");
+        }
+        p->n_ring = static_cast<int>(rings.size());
+    }
     if (rc == SDFG_OK) {
         for (int g = 0; g < n; ++g) {
             if (run_of[g] < 0 || p->on_chain[g]) continue;

@@ -29,6 +29,9 @@ struct LaunchSet {
     int k = 8;
     int warps = 8;
     int check_stride = 64;
+    // fixed-step FP32/BF16 grids only: every unit on the reassociated pipe; the
+    // caller puts each grid's ring into both of its ping-pong grids
+    bool scaled_edges = false;
 
     std::vector<PGrid> grids;
     std::vector<PState> state0;
@@ -57,8 +60,8 @@ struct LaunchSet {
 void plan_grid_passes(int t0, int steps, int T_cap, bool tol_mode, int check_stride, int k, std::vector<int> &info,
                       std::vector<int> &tend);
 
-int persistent_blocks_per_sm(int dtype, int warps);
-int launch_persistent(const PLaunch &L, int dtype, int warps, int blocks, cudaStream_t s);
+int persistent_blocks_per_sm(int dtype, int warps, bool scaled_edges);
+int launch_persistent(const PLaunch &L, int dtype, int warps, int blocks, bool scaled_edges, cudaStream_t s);
 int launch_finalize(const void *fdescs, int n, const PGrid *grids, const PState *state, int dtype, int max_rows,
                     cudaStream_t s);
 size_t final_desc_bytes();

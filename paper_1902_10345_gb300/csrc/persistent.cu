@@ -33,15 +33,15 @@ __device__ __forceinline__ bool warp_wait(Pred pred, unsigned long long timeout_
     }
 }
 
-template <class ST, int V>
+template <class ST, int V, bool SE>
 __device__ __forceinline__ bool run_depth(int k, const void *tmap, ST *dst, const GridGeo &g, int s, int q, ST *ring,
                                           uint64_t *bars, uint32_t &ctr, int res, double2 *partial,
                                           unsigned long long timeout_ns) {
     switch (k) {
-        case 1: return run_unit<ST, V, 1>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
-        case 2: return run_unit<ST, V, 2>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
-        case 4: return run_unit<ST, V, 4>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
-        default: return run_unit<ST, V, 8>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
+        case 1: return run_unit<ST, V, 1, SE>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
+        case 2: return run_unit<ST, V, 2, SE>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
+        case 4: return run_unit<ST, V, 4, SE>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
+        default: return run_unit<ST, V, 8, SE>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
     }
 }
 
@@ -49,7 +49,9 @@ __device__ __forceinline__ bool run_depth(int k, const void *tmap, ST *dst, cons
 #define SDFG_PK_MINB 3  // 128-thread CTAs per SM the register allocation must allow
 #endif
 
-template <class ST, int V>
+// SE: fixed-step FP32/BF16 grids only, every unit on the reassociated pipe (see
+// run_unit).
+template <class ST, int V, bool SE>
 __global__ void __launch_bounds__(128, SDFG_PK_MINB) persistent_kernel(const PLaunch L) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bars[MAX_WARPS][STAGES];
@@ -131,7 +133,7 @@ __global__ void __launch_bounds__(128, SDFG_PK_MINB) persistent_kernel(const PLa
             }
             __syncwarp();
             double2 *partial = res ? L.partials + static_cast<size_t>(cnum & 1) * L.total_units + unit_off + u : nullptr;
-            const bool ok = run_depth<ST, V>(info & PASS_K_MASK, tm, static_cast<ST *>(G.buf[dstb]), geo, s, q, ring,
+            const bool ok = run_depth<ST, V, SE>(info & PASS_K_MASK, tm, static_cast<ST *>(G.buf[dstb]), geo, s, q, ring,
                                              bars[warp], ctr, res, partial, L.timeout_ns);
             if (!ok) {
                 if (lane == 0) set_device_error(L.err, DEV_ERR_TIMEOUT_TMA);
@@ -222,22 +224,22 @@ __global__ void finalize_kernel(const FinalDesc *__restrict__ fd, const PGrid *_
 }
 
 // ------------------------------------------------------------- launchers ---
-template <class ST>
+template <class ST, bool SE>
 static const void *pk_fn() {
     return reinterpret_cast<const void *>(
-        &persistent_kernel<ST, Store<ST>::bytes == 8 ? 2 : (Store<ST>::bytes == 4 ? SDFG_F32_V : 4)>);
+        &persistent_kernel<ST, Store<ST>::bytes == 8 ? 2 : (Store<ST>::bytes == 4 ? SDFG_F32_V : 4), SE>);
 }
 
-static const void *persistent_fn(int dtype) {
+static const void *persistent_fn(int dtype, bool scaled_edges) {
     switch (dtype) {
-        case SDFG_F32: return pk_fn<float>();
-        case SDFG_BF16: return pk_fn<__nv_bfloat16>();
-        default: return pk_fn<double>();
+        case SDFG_F32: return scaled_edges ? pk_fn<float, true>() : pk_fn<float, false>();
+        case SDFG_BF16: return scaled_edges ? pk_fn<__nv_bfloat16, true>() : pk_fn<__nv_bfloat16, false>();
+        default: return pk_fn<double, false>();
     }
 }
 
-int persistent_blocks_per_sm(int dtype, int warps) {
-    const void *fn = persistent_fn(dtype);
+int persistent_blocks_per_sm(int dtype, int warps, bool scaled_edges) {
+    const void *fn = persistent_fn(dtype, scaled_edges);
     const size_t smem = temporal_smem_bytes(dtype, warps);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) {
         cudaGetLastError();
@@ -251,8 +253,8 @@ int persistent_blocks_per_sm(int dtype, int warps) {
     return n;
 }
 
-int launch_persistent(const PLaunch &L, int dtype, int warps, int blocks, cudaStream_t s) {
-    const void *fn = persistent_fn(dtype);
+int launch_persistent(const PLaunch &L, int dtype, int warps, int blocks, bool scaled_edges, cudaStream_t s) {
+    const void *fn = persistent_fn(dtype, scaled_edges);
     const size_t smem = temporal_smem_bytes(dtype, warps);  // attribute raised by persistent_blocks_per_sm
     PLaunch l = L;
     void *args[] = {&l};

@@ -274,6 +274,12 @@ struct NoHook {
     __device__ __forceinline__ void done(int) {}
 };
 
+// A unit of the persistent kernel's fixed-step variant: it may hold row 0 or
+// row R-1 in the reassociated pipe.
+struct EdgeHook : NoHook {
+    static constexpr bool EDGES = true;
+};
+
 // CR: rows per TMA chunk (CHUNK_ROWS; the chain kernels stream taller ones).
 template <class ST, int V, int K, bool COLCHK, bool RES, bool EXACT, int CR = CHUNK_ROWS>
 struct UnitPipe {
@@ -659,7 +665,9 @@ struct UnitPipe {
 // (source buffer), write `dst`.  res_flags bit 0: accumulate the squared
 // level-1 update (the first step of a solve), bit 1: the squared level-K
 // update (a check step).  Returns false if a TMA wait ran out.
-template <class ST, int V, int K>
+// SE (no residuals): the reassociated pipe everywhere, the boundary ring held
+// scaled and never stored (the caller has put it into both grids).
+template <class ST, int V, int K, bool SE = false>
 __device__ __forceinline__ bool run_unit(const void *tmap, ST *dst, const GridGeo &g, int strip, int seg, ST *ring,
                                          uint64_t *bars, uint32_t &chunk_ctr, int res_flags, double2 *partial,
                                          unsigned long long timeout_ns) {
@@ -688,29 +696,33 @@ __device__ __forceinline__ bool run_unit(const void *tmap, ST *dst, const GridGe
 
     bool ok;
     double ar = 0.0, ac = 0.0;
-#define SDFG_RUN_PIPE(CHK, RS, EX)                                                                          \
+#define SDFG_RUN_PIPE(CHK, RS, EX, HOOK)                                                                    \
     {                                                                                                   \
         UnitPipe<ST, V, K, CHK, RS, EX> p;                                                                  \
         p.tmap = tmap; p.dst = dst; p.ld = g.ld; p.R = g.R; p.C = g.C;                                  \
         p.X = X; p.y0 = y0; p.y1 = y1; p.rb = rb; p.n_steps = n_steps; p.n_chunks = n_chunks;           \
-        p.sy0 = y0; p.sy1 = y1;                                                                         \
+        p.sy0 = SE ? max(y0, 1) : y0; p.sy1 = SE ? min(y1, g.R - 1) : y1;                               \
         p.base = chunk_ctr; p.ring = ring; p.bars = bars; p.lane = lane;                                \
         p.colmask = colmask; p.resmask = resmask; p.own_lane = own_lane; p.full_vec = full_vec;         \
         p.res_flags = res_flags; p.timeout_ns = timeout_ns;                                             \
-        ok = p.run();                                                                                   \
+        HOOK hk;                                                                                        \
+        ok = p.run(hk);                                                                                 \
         if (RS) { ar = p.acc_ref; ac = p.acc_chk; }                                                     \
     }
     // rows rb .. y1+K-1 are read: a boundary row is among them in the first
     // and the last segments
     const bool rowedge = (rb <= 0) || (y1 + K - 1 >= g.R - 1);
-    if (res_flags) {
-        if (colchk) SDFG_RUN_PIPE(true, true, true)
-        else if (rowedge) SDFG_RUN_PIPE(false, true, true)
-        else SDFG_RUN_PIPE(false, true, false)
+    if constexpr (SE) {
+        if (colchk) SDFG_RUN_PIPE(true, false, false, EdgeHook)
+        else SDFG_RUN_PIPE(false, false, false, EdgeHook)
+    } else if (res_flags) {
+        if (colchk) SDFG_RUN_PIPE(true, true, true, NoHook)
+        else if (rowedge) SDFG_RUN_PIPE(false, true, true, NoHook)
+        else SDFG_RUN_PIPE(false, true, false, NoHook)
     } else {
-        if (colchk) SDFG_RUN_PIPE(true, false, true)
-        else if (rowedge) SDFG_RUN_PIPE(false, false, true)
-        else SDFG_RUN_PIPE(false, false, false)
+        if (colchk) SDFG_RUN_PIPE(true, false, true, NoHook)
+        else if (rowedge) SDFG_RUN_PIPE(false, false, true, NoHook)
+        else SDFG_RUN_PIPE(false, false, false, NoHook)
     }
 #undef SDFG_RUN_PIPE
     chunk_ctr += static_cast<uint32_t>(n_chunks);
