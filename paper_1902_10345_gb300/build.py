@@ -60,8 +60,8 @@ def _digest() -> str:
 
 
 KERNEL_FILES = ["device_common.cuh", "temporal_unit.cuh", "geometry.h", "persistent.h", "persistent.cu", "kernels.cu"]
-KERNEL_FILES_3D = ["device_common.cuh", "jacobi3d.cu"]
-KERNEL_FILES_SOR = ["device_common.cuh", "sor2d.cu"]
+KERNEL_FILES_3D = ["device_common.cuh", "jacobi3d.cu", "jacobi3d.h", "jacobi3d_fused.cu"]
+KERNEL_FILES_SOR = ["device_common.cuh", "sor2d.cu", "sor_row.cuh"]
 KERNEL_FILES_RESIDENT = ["device_common.cuh", "resident.cu"]
 KERNEL_FILES_CHAIN = ["device_common.cuh", "temporal_unit.cuh", "geometry.h", "chain.cuh", "skewed.cu", "chain_batch.cu"]
 
