@@ -63,6 +63,7 @@ KERNEL_FILES = ["device_common.cuh", "temporal_unit.cuh", "geometry.h", "persist
 KERNEL_FILES_3D = ["device_common.cuh", "jacobi3d.cu", "jacobi3d.h", "jacobi3d_fused.cu"]
 KERNEL_FILES_SOR = ["device_common.cuh", "sor2d.cu", "sor_row.cuh"]
 KERNEL_FILES_RESIDENT = ["device_common.cuh", "resident.cu"]
+KERNEL_FILES_TILES = ["device_common.cuh", "exchange.cuh", "sor_row.cuh", "tiles.h", "tiles.cuh"]
 KERNEL_FILES_CHAIN = ["device_common.cuh", "temporal_unit.cuh", "geometry.h", "chain.cuh", "skewed.cu", "chain_batch.cu"]
 
 
