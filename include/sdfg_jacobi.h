@@ -364,7 +364,8 @@ int sdfg_sor2d(const void *in, void *out, int rows, int cols, int ld, int T, dou
  * calling stream (min(T, 64) steps each: the streamed and persistent kernels
  * at k = 2, 4, 8 and several segment heights, plus the register-resident
  * kernel at k = 2, 4, 8 for FP32/BF16 grids whose two buffers fit in
- * 96 MiB), caches the best by shape class, and returns it.  Allocates two
+ * 96 MiB, and what an untuned call runs, which is returned as kernel 0), caches
+ * the best by shape class, and returns it.  Allocates two
  * scratch grids for the trials and frees them. */
 int sdfg_autotune(int rows, int cols, int T, int dtype, sdfg_config *best, void *stream);
 

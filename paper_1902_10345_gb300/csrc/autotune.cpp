@@ -13,7 +13,6 @@
 #include <vector>
 
 #include "runtime.h"
-#include "tiles.h"
 
 namespace sdfg {
 
@@ -122,9 +121,8 @@ extern "C" int sdfg_autotune(int rows, int cols, int T, int dtype, sdfg_config *
             if (L <= 2 * rows) cands.push_back(sdfg_config{SDFG_KERNEL_SKEWED, k, L, 4});
         if (try_resident) cands.push_back(sdfg_config{SDFG_KERNEL_RESIDENT, k, 0, 0});
     }
-    // what an untuned call runs where the chip's registers hold the grid
-    TilePlan plan;
-    if (plan_tiles(rows, cols, dtype, st->sm_count, &plan)) cands.push_back(sdfg_config{SDFG_KERNEL_AUTO, 0, 0, 0});
+    // what an untuned call runs (tiles, chains by the grid's size, FP64 paths)
+    cands.push_back(sdfg_config{SDFG_KERNEL_AUTO, 0, 0, 0});
     float best_ms = 1e30f;
     sdfg_config winner = {SDFG_KERNEL_TEMPORAL, default_depth(dtype), 0, 4};
     for (const sdfg_config &c : cands) {
