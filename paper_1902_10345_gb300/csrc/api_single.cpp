@@ -217,7 +217,7 @@ int run_single(const void *in, void *out, int R, int C, int ld, long long T, int
             if (rc != SDFG_OK || ran) return rc;
         }
         TilePlan plan;
-        if (plan_tiles(R, C, dtype, st->sm_count, &plan)) {
+        if (plan_tiles(R, C, dtype, st, &plan)) {
             rc = run_tiles(in, out, R, C, ld, T, dtype, plan, st, s);
             if (rc != SDFG_ERR_NOMEM) return rc;
         }

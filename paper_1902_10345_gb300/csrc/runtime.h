@@ -120,8 +120,8 @@ int run_resident_passes(const void *src0, void *first, void *second, const std::
 
 // ---- register tiles (tiles.cu) --------------------------------------------------
 struct TilePlan;  // tiles.h
-// The kernel variant and tile counts for a grid (FP32/BF16); false if it does not fit the chip's registers.
-bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan, bool sor = false);
+// The kernel variant and tile counts for a grid (FP32/BF16) on the current device `st`; false if it does not fit the chip's registers.
+bool plan_tiles(int R, int C, int dtype, const DeviceState *st, TilePlan *plan, bool sor = false);
 // T >= 1 steps in one cooperative launch with that plan; any ld and alignment, in == out allowed.
 // omega: T red-black SOR iterations instead (a plan made for them).
 int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int dtype, const TilePlan &plan,

@@ -476,7 +476,7 @@ extern "C" int sdfg_sor2d(const void *in, void *out, int rows, int cols, int ld,
     // 1500^2 261 -> 230, 1800^2 311 -> 355; T=8: 1000^2 18 -> 23.
     if (dtype != SDFG_F64 && T >= 32 && static_cast<long long>(rows) * cols <= 2400000) {
         TilePlan plan;
-        if (plan_tiles(rows, cols, dtype, st->sm_count, &plan, true)) {
+        if (plan_tiles(rows, cols, dtype, st, &plan, true)) {
             rc = run_tiles(in, out, rows, cols, ld, T, dtype, plan, st, s, &omega);
             if (rc != SDFG_ERR_NOMEM) return rc;
         }

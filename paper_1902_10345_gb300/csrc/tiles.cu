@@ -2,9 +2,9 @@
 #include <string.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "launchset.h"
+#include "per_device.h"
 #include "tiles.cuh"
 
 namespace sdfg {
@@ -32,23 +32,21 @@ const void *tile_fn(TileShape v, int dtype, bool sor) {
     }
 }
 
-// CTAs of variant `i` an SM holds (a property of the compiled kernel)
-int tile_blocks_per_sm(int i, int dtype, bool sor) {
-    static std::mutex mu;
-    static int cache[kShapeCount][2][2];
-    std::lock_guard<std::mutex> lk(mu);
-    int &n = cache[i][dtype == SDFG_BF16][sor];
-    if (n == 0) {
+// CTAs of variant `i` an SM holds (a property of the compiled kernel), and the
+// kernel's shared-memory limit raised: both on the current device, which is `device`
+int tile_blocks_per_sm(int i, int dtype, bool sor, int device) {
+    static PerDevice<kShapeCount * 4> known;
+    return known.get(device, (i * 2 + (dtype == SDFG_BF16)) * 2 + sor, [&]() {
         const TileShape v = kShapes[i];
         const void *fn = tile_fn(v, dtype, sor);
+        int n = 0;
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(tile_smem(v))) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, 32 * v.nw, tile_smem(v)) != cudaSuccess) {
             cudaGetLastError();
-            n = 0;
             return 0;
         }
-    }
-    return n;
+        return n;
+    });
 }
 
 // Tiles along an axis of n points when a tile answers for t of them.
@@ -74,7 +72,8 @@ template <class First> bool halos_in_neighbours(int n, int extent, int tile, int
 // neighbouring band's row.  Measured best and chosen: 256^2 T=100 8 warps x 4
 // rows (50 us; 7 rows 54, 16 x 4 60), 1301 x 1777 T=150 16 x 12 (146 us) and
 // 16 x 11 (148), 2048^2 T=1024 16 x 17 (1345 us; 16 x 18 1450).
-bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan, bool sor) {
+bool plan_tiles(int R, int C, int dtype, const DeviceState *st, TilePlan *plan, bool sor) {
+    const int sm_count = st->sm_count;
     if (dtype == SDFG_F64 || R < 3 || C < 3) return false;
     const int x = tiles_along(C, TK_TX);
     if (x > 4LL * sm_count) return false;
@@ -89,7 +88,7 @@ bool plan_tiles(int R, int C, int dtype, int sm_count, TilePlan *plan, bool sor)
         const long long n = static_cast<long long>(x) * y;
         if (n > 4LL * sm_count || !halos_in_neighbours(y, R, TY, TK_HALO, [&](int t) { return tile_y0_of(R, y, t, TY); }))
             continue;
-        if (n > static_cast<long long>(tile_blocks_per_sm(i, dtype, sor)) * sm_count) continue;
+        if (n > static_cast<long long>(tile_blocks_per_sm(i, dtype, sor, st->device)) * sm_count) continue;
         const int per_sm = static_cast<int>((n + sm_count - 1) / sm_count);
         const double cost = 8.0 * (14.0 * v.rb * (v.nw / 4) * per_sm + 250.0);
         if (best == 0.0 || cost < best) {
