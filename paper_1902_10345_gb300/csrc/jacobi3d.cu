@@ -281,11 +281,8 @@ static size_t j3_smem(int dtype) { return static_cast<size_t>(J3_NS) * J3_BY * j
 static int launch_j3(const CUtensorMap &tm, void *dst, const J3Geo &g, int dtype, int *err, cudaStream_t s) {
     const void *fn = j3_kernel(dtype);
     const size_t smem = j3_smem(dtype);
-    static bool attr_done[3] = {false, false, false};
-    if (!attr_done[dtype]) {
-        SDFG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        attr_done[dtype] = true;
-    }
+    int rc = raise_smem_limit(fn, smem);
+    if (rc != SDFG_OK) return rc;
     CUtensorMap t = tm;
     J3Geo gg = g;
     void *dp = dst;

@@ -372,7 +372,8 @@ J3FGeo j3_fused_plan(int K, int D, int R, int C, int ld, int dtype, int sm_count
 int launch_j3_fused(const CUtensorMap &tm, void *dst, const J3FGeo &g, int K, int dtype, int *err, cudaStream_t s) {
     const void *fn = fused_fn(K, dtype);
     const size_t smem = static_cast<size_t>(JF_NS) * j3_fused_rows(K) * 128 * dtype_bytes(dtype);
-    SDFG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    int rc = raise_smem_limit(fn, smem);
+    if (rc != SDFG_OK) return rc;
     double f = 1.0;
     for (int i = 0; i < K; ++i) f /= 7.0;
     float hi = static_cast<float>(f), lo = static_cast<float>(f - static_cast<double>(hi));

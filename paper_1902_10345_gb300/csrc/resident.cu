@@ -367,15 +367,10 @@ int run_resident_passes(const void *src0, void *first, void *second, const std::
         if (k < 1 || k > RS_HALO) return set_error(SDFG_ERR_INVAL, "resident kernel: k=%d outside 1..%d", k, RS_HALO);
     const void *fn = resident_fn(dtype);
     const size_t smem = static_cast<size_t>(RS_BY) * RS_W * dtype_bytes(dtype);
-    static bool attr_done[2] = {false, false};
-    const int slot = dtype == SDFG_BF16 ? 1 : 0;
-    if (!attr_done[slot]) {
-        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) return cuda_error(e, "resident attribute");
-        attr_done[slot] = true;
-    }
+    int rc = raise_smem_limit(fn, smem);
+    if (rc != SDFG_OK) return rc;
     alignas(128) CUtensorMap tm_src0, tm_first, tm_second;
-    int rc = encode_tmap3d(&tm_src0, src0, dtype, 1, R, C, ld, RS_W, RS_BOX_ROWS);
+    rc = encode_tmap3d(&tm_src0, src0, dtype, 1, R, C, ld, RS_W, RS_BOX_ROWS);
     if (rc == SDFG_OK) rc = encode_tmap3d(&tm_first, first, dtype, 1, R, C, ld, RS_W, RS_BOX_ROWS);
     if (rc == SDFG_OK) rc = encode_tmap3d(&tm_second, second, dtype, 1, R, C, ld, RS_W, RS_BOX_ROWS);
     if (rc != SDFG_OK) return rc;

@@ -7,7 +7,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <map>
 #include <string>
+#include <utility>
 
 namespace sdfg {
 
@@ -63,6 +65,19 @@ int current_device(DeviceState **st) {
         return set_error(SDFG_ERR_UNSUPPORTED, "device %d is sm_%d%d; this library is built for sm_103a only", dev,
                          d.major, d.minor);
     *st = &d;
+    return SDFG_OK;
+}
+
+int raise_smem_limit(const void *fn, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, size_t> limit;  // per device and kernel
+    int dev = -1;
+    SDFG_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    size_t &have = limit[{dev, fn}];
+    if (have >= bytes) return SDFG_OK;
+    SDFG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)));
+    have = bytes;
     return SDFG_OK;
 }
 

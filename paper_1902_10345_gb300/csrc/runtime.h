@@ -39,6 +39,10 @@ struct DeviceState {
 // SDFG_ERR_UNSUPPORTED when the device is not an sm_103 part.
 int current_device(DeviceState **st);
 
+// Raises a kernel's dynamic shared-memory limit on the current device, where it
+// holds; once per device and kernel.
+int raise_smem_limit(const void *fn, size_t bytes);
+
 // ---- dtype -------------------------------------------------------------------
 inline bool dtype_valid(int dt) { return dt == SDFG_F32 || dt == SDFG_BF16 || dt == SDFG_F64; }
 inline int dtype_bytes(int dt) { return dt == SDFG_F64 ? 8 : (dt == SDFG_BF16 ? 2 : 4); }

@@ -518,12 +518,7 @@ extern "C" int sdfg_sor2d(const void *in, void *out, int rows, int cols, int ld,
     }
     const void *fn = sor_kernel(dtype);
     const size_t smem = static_cast<size_t>(box_rows) * box_cols * S;
-    static bool attr_done[3] = {false, false, false};
-    if (!attr_done[dtype]) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) rc = cuda_error(e, "sor2d attribute");
-        else attr_done[dtype] = true;
-    }
+    if (rc == SDFG_OK) rc = raise_smem_limit(fn, smem);
     alignas(128) CUtensorMap tm_src0, tm_first, tm_second;
     if (rc == SDFG_OK) rc = encode_tmap3d(&tm_src0, src0, dtype, 1, rows, cols, ldw, box_cols, box_rows);
     if (rc == SDFG_OK) rc = encode_tmap3d(&tm_first, first, dtype, 1, rows, cols, ldw, box_cols, box_rows);
