@@ -25,27 +25,30 @@
 namespace sdfg {
 
 // ---------------------------------------------------------------- copies ----
+// A block column per grid, more grids than the launch is high (65535 at most) in turn.
 template <class ST>
-__global__ void ring_copy_kernel(const RingCopy *__restrict__ descs) {
-    const RingCopy r = descs[blockIdx.y];
-    const int n = 2 * r.C + 2 * max(r.R - 2, 0);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        int row, col;
-        if (i < r.C) {
-            row = 0;
-            col = i;
-        } else if (i < 2 * r.C) {
-            row = r.R - 1;
-            col = i - r.C;
-        } else {
-            const int t = i - 2 * r.C;
-            row = 1 + (t >> 1);
-            col = (t & 1) ? r.C - 1 : 0;
+__global__ void ring_copy_kernel(const RingCopy *__restrict__ descs, int n_descs) {
+    for (int d = blockIdx.y; d < n_descs; d += gridDim.y) {
+        const RingCopy r = descs[d];
+        const int n = 2 * r.C + 2 * max(r.R - 2, 0);
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+            int row, col;
+            if (i < r.C) {
+                row = 0;
+                col = i;
+            } else if (i < 2 * r.C) {
+                row = r.R - 1;
+                col = i - r.C;
+            } else {
+                const int t = i - 2 * r.C;
+                row = 1 + (t >> 1);
+                col = (t & 1) ? r.C - 1 : 0;
+            }
+            const size_t at = static_cast<size_t>(row) * r.ld + col;
+            const ST v = static_cast<const ST *>(r.src)[at];
+            if (r.dst[0]) static_cast<ST *>(r.dst[0])[at] = v;
+            if (r.dst[1]) static_cast<ST *>(r.dst[1])[at] = v;
         }
-        const size_t at = static_cast<size_t>(row) * r.ld + col;
-        const ST v = static_cast<const ST *>(r.src)[at];
-        if (r.dst[0]) static_cast<ST *>(r.dst[0])[at] = v;
-        if (r.dst[1]) static_cast<ST *>(r.dst[1])[at] = v;
     }
 }
 
@@ -61,12 +64,12 @@ __global__ void grid_copy_kernel(const GridCopy *__restrict__ descs) {
 
 int launch_ring_copy(const RingCopy *d_descs, int n, int max_ring, int dtype, cudaStream_t s) {
     if (n <= 0) return SDFG_OK;
-    const dim3 grid(static_cast<unsigned>(std::min(std::max((max_ring + 255) / 256, 1), 64)), static_cast<unsigned>(n));
+    const dim3 grid(static_cast<unsigned>(std::min(std::max((max_ring + 255) / 256, 1), 64)), static_cast<unsigned>(std::min(n, 65535)));
     TimedLaunch t = stats_begin(FAM_COPY, s);
     switch (dtype) {
-        case SDFG_F32: ring_copy_kernel<float><<<grid, 256, 0, s>>>(d_descs); break;
-        case SDFG_BF16: ring_copy_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(d_descs); break;
-        default: ring_copy_kernel<double><<<grid, 256, 0, s>>>(d_descs); break;
+        case SDFG_F32: ring_copy_kernel<float><<<grid, 256, 0, s>>>(d_descs, n); break;
+        case SDFG_BF16: ring_copy_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(d_descs, n); break;
+        default: ring_copy_kernel<double><<<grid, 256, 0, s>>>(d_descs, n); break;
     }
     stats_end(t, s);
     SDFG_CUDA(cudaGetLastError());
