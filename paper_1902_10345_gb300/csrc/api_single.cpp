@@ -36,7 +36,8 @@ int validate_grid(const void *in, const void *out, int R, int C, int ld, long lo
     return SDFG_OK;
 }
 
-int resolve_config(const sdfg_config *cfg, int R, int C, int dtype, sdfg_config *out) {
+// use_tuned: what the autotuner chose for the shape's class counts (not for its own trials).
+int resolve_config(const sdfg_config *cfg, int R, int C, int dtype, bool use_tuned, sdfg_config *out) {
     sdfg_config c = {SDFG_KERNEL_AUTO, 0, 0, 0};
     if (cfg) c = *cfg;
     if (c.kernel < SDFG_KERNEL_AUTO || c.kernel > SDFG_KERNEL_SKEWED)
@@ -45,7 +46,7 @@ int resolve_config(const sdfg_config *cfg, int R, int C, int dtype, sdfg_config 
     if (c.seg_rows < 0 || c.warps < 0 || c.warps > MAX_WARPS)
         return set_error(SDFG_ERR_INVAL, "bad seg_rows/warps (%d/%d)", c.seg_rows, c.warps);
     sdfg_config tuned;
-    const bool have = autotune_lookup(R, C, dtype, &tuned) && tuned.kernel != SDFG_KERNEL_AUTO;
+    const bool have = use_tuned && autotune_lookup(R, C, dtype, &tuned) && tuned.kernel != SDFG_KERNEL_AUTO;
     // large grids: one launch for all passes (no per-pass tail) -- the chain
     // kernel -- for FP32/BF16 storage; one step per launch for FP64, which the
     // FP64 pipe bounds, so that fused steps only recompute halos (2048^2 T=20
@@ -192,16 +193,16 @@ static int run_single_persistent(const void *in, void *out, int R, int C, int ld
 }
 
 // Core single-grid run.  in_disposable: `in` may be overwritten (it then
-// serves as the scratch grid).
+// serves as the scratch grid).  use_tuned: see resolve_config.
 int run_single(const void *in, void *out, int R, int C, int ld, long long T, int dtype, const sdfg_config *cfg,
-               bool in_disposable, cudaStream_t s) {
+               bool in_disposable, cudaStream_t s, bool use_tuned = true) {
     if (R == 0 || C == 0) return SDFG_OK;
     DeviceState *st = nullptr;
     int rc = current_device(&st);
     if (rc != SDFG_OK) return rc;
     if (T == 0 || R < 3 || C < 3) return launch_copy2d(out, ld, in, ld, R, C, dtype, s);
     sdfg_config c;
-    rc = resolve_config(cfg, R, C, dtype, &c);
+    rc = resolve_config(cfg, R, C, dtype, use_tuned, &c);
     if (rc != SDFG_OK) return rc;
     // nothing asked for, and nothing else tuned: a grid that the chip's
     // registers hold runs there from the first step to the last.  Measured
@@ -210,7 +211,7 @@ int run_single(const void *in, void *out, int R, int C, int ld, long long T, int
     // 2048^2 T=1024 1345 us (6676, chains; 1610 with register-resident passes)
     sdfg_config tuned;
     if ((!cfg || (cfg->kernel == SDFG_KERNEL_AUTO && cfg->k == 0 && cfg->seg_rows == 0 && cfg->warps == 0)) &&
-        (!autotune_lookup(R, C, dtype, &tuned) || tuned.kernel == SDFG_KERNEL_AUTO)) {
+        (!use_tuned || !autotune_lookup(R, C, dtype, &tuned) || tuned.kernel == SDFG_KERNEL_AUTO)) {
         if (dtype == SDFG_F64) {
             bool ran = false;
             rc = run_tiles64(in, out, R, C, ld, T, st, s, &ran);
@@ -286,7 +287,7 @@ int run_single_with_scratch(const void *in, void *out, void *scratch, int R, int
     if (R == 0 || C == 0) return SDFG_OK;
     if (T == 0 || R < 3 || C < 3) return launch_copy2d(out, ld, in, ld, R, C, dtype, s);
     sdfg_config c;
-    int rc = resolve_config(cfg, R, C, dtype, &c);
+    int rc = resolve_config(cfg, R, C, dtype, true, &c);
     if (rc != SDFG_OK) return rc;
     if (c.kernel != SDFG_KERNEL_NAIVE) c.kernel = SDFG_KERNEL_TEMPORAL;
     const std::vector<int> ks = c.kernel == SDFG_KERNEL_NAIVE ? std::vector<int>(1, static_cast<int>(T))

@@ -17,7 +17,7 @@
 namespace sdfg {
 
 int run_single(const void *in, void *out, int R, int C, int ld, long long T, int dtype, const sdfg_config *cfg,
-               bool in_disposable, cudaStream_t s);
+               bool in_disposable, cudaStream_t s, bool use_tuned);
 
 namespace {
 using Key = std::tuple<int, int, int>;
@@ -126,11 +126,11 @@ extern "C" int sdfg_autotune(int rows, int cols, int T, int dtype, sdfg_config *
     float best_ms = 1e30f;
     sdfg_config winner = {SDFG_KERNEL_TEMPORAL, default_depth(dtype), 0, 4};
     for (const sdfg_config &c : cands) {
-        // warm-up, then timed
-        rc = run_single(a, b, rows, cols, ld, Tp, dtype, &c, false, s);
+        // warm-up, then timed; no trial sees what an earlier call chose for the class
+        rc = run_single(a, b, rows, cols, ld, Tp, dtype, &c, false, s, false);
         if (rc != SDFG_OK) break;
         cudaEventRecord(e0, s);
-        rc = run_single(a, b, rows, cols, ld, Tp, dtype, &c, false, s);
+        rc = run_single(a, b, rows, cols, ld, Tp, dtype, &c, false, s, false);
         cudaEventRecord(e1, s);
         if (rc != SDFG_OK) break;
         if (cudaEventSynchronize(e1) != cudaSuccess) {
