@@ -260,7 +260,8 @@ int sdfg_jacobi2d_batch(sdfg_desc *desc, int n, int check_stride, void *stream);
  * grids (tol = 0) of at least 2^20 points run as skewed chains of 512 rows
  * at the library's depth (8 for FP32/BF16, 4 for FP64) in one launch, every
  * other grid on the persistent kernel as above in a second launch; NULL: the
- * batch autotuner's cached choice for this class of batch, else the
+ * batch autotuner's cached choice for this class of batch, else, as with every
+ * field 0, the
  * persistent kernel (a fixed-step FP32 or BF16 batch of 2^18 points or more
  * with depth and segment height by its size and every unit reassociated).
  * Chains pay off for grids whose own work is long
@@ -373,7 +374,8 @@ int sdfg_autotune(int rows, int cols, int T, int dtype, sdfg_config *best, void 
  * are overwritten by the trial runs): the persistent kernel at k = 4, 8 and
  * several segment heights, and, when no grid has tol > 0, the chain kernel at
  * k = 4, 8 for the large grids and the persistent kernel at 128- or 256-row
- * segments for the others; caches the best for batches of this
+ * segments for the others, and what an untuned plan runs, which is returned as
+ * kernel 0; caches the best for batches of this
  * class (dtype, grid count, mean area), and returns it.  Plans created
  * afterwards with cfg == NULL for a batch of the same class use it. */
 int sdfg_autotune_batch(const sdfg_desc *desc, int n, int check_stride, sdfg_config *best, void *stream);

@@ -393,19 +393,19 @@ static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int c
         any_tol |= d.tol > 0.0;
     }
     if (any_tol && check_stride < 1) return set_error(SDFG_ERR_INVAL, "batch: check_stride must be >= 1");
-    sdfg_config c = {SDFG_KERNEL_PERSISTENT, 0, 0, 0};
-    bool scaled_edges = false;
-    if (cfg) {
+    // all zero (asked for, tuned, or nothing tuned): the library's own choice
+    sdfg_config c = {SDFG_KERNEL_AUTO, 0, 0, 0};
+    double area = 0.0;
+    for (int g = 0; g < n; ++g) area += static_cast<double>(desc[g].rows) * desc[g].cols;
+    area /= std::max(n, 1);
+    if (cfg)
         c = *cfg;
-    } else if (n > 0) {
-        double area = 0.0;
-        for (int g = 0; g < n; ++g) area += static_cast<double>(desc[g].rows) * desc[g].cols;
-        area /= n;
-        sdfg_config tuned;
-        if (autotune_lookup(-n, -static_cast<int>(area > 2e9 ? 2e9 : area), dtype, &tuned))
-            c = tuned;
-        else if (!any_tol)
-            scaled_edges = untuned_batch(area * n, n, dtype, &c);
+    else if (n > 0)
+        autotune_lookup(-n, -static_cast<int>(area > 2e9 ? 2e9 : area), dtype, &c);
+    bool scaled_edges = false;
+    if (c.kernel == SDFG_KERNEL_AUTO && c.k == 0 && c.seg_rows == 0 && c.warps == 0) {
+        c.kernel = SDFG_KERNEL_PERSISTENT;
+        if (n > 0 && !any_tol) scaled_edges = untuned_batch(area * n, n, dtype, &c);
     }
     if (c.k != 0 && !depth_supported(c.k)) return set_error(SDFG_ERR_INVAL, "batch: k must be 1, 2, 4 or 8");
     if (c.warps < 0 || c.warps > MAX_WARPS || c.seg_rows < 0) return set_error(SDFG_ERR_INVAL, "batch: bad config");
@@ -718,9 +718,9 @@ extern "C" int sdfg_jacobi2d_solve(sdfg_desc *desc, int check_stride, const sdfg
 
 // ---------------------------------------------------------- batch tuner -----
 // Candidates: the persistent kernel at fused depth k in {4, 8} x segment
-// height in {96, 128, 192, 256, 384}, and, when no grid solves to a
-// tolerance, the hybrid (large grids on the chain kernel) at k in {4, 8} x
-// segment height in {128, 256}.
+// height in {96, 128, 192, 256, 384}, when no grid solves to a
+// tolerance the hybrid (large grids on the chain kernel) at k in {4, 8} x
+// segment height in {128, 256}, and what an untuned plan runs (kernel AUTO).
 // Each is built as a plan over the caller's batch, run once to warm up and
 // once timed; the fastest is cached under the batch's class (dtype, grid
 // count and mean area, both power-of-two buckets) and returned.
@@ -744,6 +744,7 @@ extern "C" int sdfg_autotune_batch(const sdfg_desc *desc, int n, int check_strid
         if (!any_tol)
             for (int seg : {128, 256}) cands.push_back(sdfg_config{SDFG_KERNEL_SKEWED, k, seg, 4});
     }
+    cands.push_back(sdfg_config{SDFG_KERNEL_AUTO, 0, 0, 0});
     float best_ms = 1e30f;
     sdfg_config winner = {SDFG_KERNEL_PERSISTENT, default_depth(dtype), 96, 4};
     std::vector<sdfg_desc> tmp(desc, desc + n);

@@ -33,3 +33,31 @@ binding.sdfg_autotune(256, 256, 8, binding.SDFG_F64, torch.cuda.current_stream()
 print(binding.sdfg_stats_get("resident")[0])
 """)
     assert out == ["2"]  # warm-up and timed run
+
+
+BATCH = """
+xs = [torch.rand((400, 400), device='cuda') for _ in range(8)]
+ys = [torch.empty_like(x) for x in xs]
+descs = [binding.desc_for(x, y, 16) for x, y in zip(xs, ys)]
+torch.cuda.synchronize()
+binding.sdfg_stats_enable(True)
+"""
+
+
+def test_retuning_a_batch_times_the_untuned_plan(tmp_path):
+    """Aligned grids below the chain kernel's size: only the untuned plan copies
+    rings, so the copies' count tells that it is a candidate."""
+    out, cache = child(tmp_path, "0 -4 -18 3 8 96 4", BATCH + """
+best = binding.sdfg_autotune_batch(descs, 64)
+print(binding.sdfg_stats_get("copy")[0], best.kernel, best.k, best.seg_rows, best.warps)
+""")
+    assert out[0] == "2"  # warm-up and timed run
+    assert cache == ["0", "-4", "-18"] + out[1:]
+
+
+def test_a_cached_untuned_choice_is_the_untuned_plan(tmp_path):
+    out, _ = child(tmp_path, "0 -4 -18 0 0 0 0", BATCH + """
+binding.check(binding.sdfg_jacobi2d_batch(descs, 64))
+print(binding.sdfg_stats_get("copy")[0])
+""")
+    assert out == ["1"]
