@@ -30,13 +30,18 @@
  *     quarter of the FP32 work and is more accurate against FP64, not less.
  *     The chain kernel and the register tiles reassociate everywhere, and so
  *     do the fused passes of the 3-D stencil (sums scaled by 7^-k).
- *     FP32 results are therefore bit-identical for the same geometry (fused
- *     depth k and segment height, hence alone or in any batch or server mix),
- *     and agree with other geometries to within the FP32 tolerance (max-abs
- *     1e-4 on fields in [0, 1]) rather than bit for bit.
+ *     FP32 results are therefore bit-identical for the same configuration
+ *     (kernel, fused depth k and segment height, hence alone or in any batch or
+ *     server mix), and agree with other configurations to within the FP32
+ *     tolerance (max-abs 1e-4 on fields in [0, 1]) rather than bit for bit.
+ *     A batch without a configuration runs one of three ways, chosen for the
+ *     batch as a whole (see the batch plans), which differ by that tolerance;
+ *     among batches that run the same way a grid's result does not depend on
+ *     its companions.  Give a configuration for the same bits in any mix.
  *   - BF16 storage: the steps fused into one pass stay in FP32 registers and
  *     values are rounded to BF16 each time a pass writes the grid, so the
  *     result also depends on k; the register tiles round once, at the end.
+ *     Batches without a configuration run at k = 8.
  *
  * Storage types: FP32 (arithmetic FP32), BF16 (the grid is stored in BF16;
  * arithmetic is FP32, and the steps fused into one pass stay in FP32
@@ -261,9 +266,11 @@ int sdfg_jacobi2d_batch(sdfg_desc *desc, int n, int check_stride, void *stream);
  * at the library's depth (8 for FP32/BF16, 4 for FP64) in one launch, every
  * other grid on the persistent kernel as above in a second launch; NULL: the
  * batch autotuner's cached choice for this class of batch, else, as with every
- * field 0, the
- * persistent kernel (a fixed-step FP32 or BF16 batch of 2^18 points or more
- * with depth and segment height by its size and every unit reassociated).
+ * field 0, the persistent kernel, one of three ways chosen for the batch by
+ * its type, points, grids and longest run: exact order at the ring, k = 8 and
+ * 96-row segments (FP64 at k = 4; every batch with a grid that solves to a
+ * tolerance, every one of less than 2^18 points), or, FP32 and BF16, every unit
+ * reassociated at k = 8 or, FP32 alone, at k = 4.
  * Chains pay off for grids whose own work is long
  * (measured on 16 grids of 2048^2, 496 steps: 5064 against 3321 GUpdates/s);
  * on the uneven 512-grid batch the persistent kernel is faster.

@@ -342,37 +342,50 @@ static void plan_free(sdfg_batch_plan *p) {
     delete p;
 }
 
-// How an untuned fixed-step batch of n grids and `points` points runs: fused
-// depth, segment height, and (the result) whether every unit takes the
-// reassociated pipe, the ring held scaled -- an eighth of the error against FP64
-// of exact-order boundary units, and fewer pipe variants in flight.
-// - Below 2^18 points, FP64, and for BF16 between 3 M and 12 M points and for
-//   large batches of small grids: as a batch with tolerance grids, depth 8, 96
-//   rows, exact order at the ring.
-// - Below 12 M points the lag from pass to pass counts: depth 8, 64 rows.
-// - From there on the warps in flight (12 per SM, 112 columns each) have several
-//   units a pass: units as tall as a third of the rows a warp has to itself
-//   (fewer halo rows), FP32 at depth 4 (which loses 2 to 7% to depth 8 on some
-//   batches and wins 20% on 384 grids of 64..512); BF16 keeps the depth, as its
-//   values are rounded once a pass.
-// Measured, ms, before -> now (points; grids of 64..2048 if not said): FP32 512
-// grids (157 M) 30.6 -> 15.1, 256 (83 M) 16.6 -> 8.9, 128 (44 M) 9.6 -> 5.6, 64
-// (22 M) 5.9 -> 3.5, 384 of 64..512 (18 M) 5.7 -> 3.8, 32 (9 M) 2.9 -> 1.9, 16
-// (2 M) 2.0 -> 1.45, 12 of 64..300 (0.3 M) 1.5 -> 1.2; BF16 157 M 32.7 -> 23.8,
-// 44 M 10.4 -> 8.8, 2 M 2.1 -> 1.5, but 384 of 64..512 6.3 -> 6.8, 128 of them
-// (6 M) 3.1 -> 3.4, so those stay.
-static bool untuned_batch(double points, int n, int dtype, sdfg_config *c) {
+// How an untuned fixed-step batch of n grids, `points` points and at most
+// `steps` steps runs: whether every unit takes the reassociated pipe, the ring held
+// scaled (the result) -- a fiftieth of the error against 64 bits of exact-order
+// boundary units, and fewer pipe variants in flight -- at which depth, and with
+// which segments.  The segments' height changes no bit of such a grid, so a grid's
+// result differs between batches that run a different one of the three ways (exact
+// order at the ring, this at depth 8, this at depth 4), and with no other companions.
+// Exact order at the ring:
+// - FP64, and below 2^18 points, where a pass is one unit's latency either way;
+// - less than 2^12 points a grid: ms, exact and this, 2000 FP32 grids of 16..64, T=
+//   50..500: 1.65, 2.14;
+// - fewer than 8 steps and 12 M points (BF16 5 M) or more, a short pass or two beside
+//   which the rings' copies count: 512 FP32 grids of 64..2048, T=1 0.24, 0.29; T=4 0.30, 0.31;
+//   16 of 64..600, T=4: 30 us, 26; BF16 32 of 64..2048, T=4: 38, 47;
+// - BF16, 5 M points or more in grids of less than 2^17: 128 grids of 64..512, T=50..
+//   500: 3.0, 3.3 ms; 384 of them 6.2, 6.4, T=7..8 219, 296 us.
+// Depth 4, for FP32 alone, whose values are not rounded between passes: 12 M points
+// or more in small grids or short runs, where the remainder passes of depth 8 bring
+// more pipe variants in flight: 384 grids of 64..512, T=50..500: depth 8 4.7 ms, 4 3.7;
+// T=13..16 339, 239 us; but 512 of 64..2048, T=50..500: 15.3, 15.8.
+// Segments by the rows that a warp in flight (12 per SM, 112 columns each) has to
+// itself in a pass: few, and the lag from pass to pass counts, many, and the halo
+// rows do; BF16 units move half the bytes and gain from fewer halo rows sooner.
+// Measured at depth 8, ms, T=50..500, grids of 64..2048 if not said, exact and at 64,
+// 128, 256 rows: FP32 32 grids (12 M points) 3.7, 2.3, 2.9, 4.6; 128 (51 M) 9.9, 6.4,
+// 5.7, 6.4; 512 (170 M) 32.3, 21.6, 17.3, 16.1 (384 rows 16.3); 16 of 64..600 (1 M)
+// 2.2, 1.6, 2.5, 4.3; BF16 64 of 64..512 (3 M) 2.5, 2.1, 2.8, 4.4; 32 4.1, 4.1, 3.6,
+// 4.9; 128 10.7, 10.6, 9.2, 9.1 (T=7..8 0.32, -, 0.28, 0.34); 512 34.6, 36, 29.3, 25.6
+// (384 rows 24.0).
+static bool untuned_batch(double points, int n, int steps, int dtype, int sm_count, sdfg_config *c) {
     const bool bf16 = dtype == SDFG_BF16;
-    if (dtype == SDFG_F64 || points < (1 << 18)) return false;
-    if (points < 12e6) {
-        if (bf16 && points >= 3e6) return false;
-        c->seg_rows = 64;
-        return true;
+    const double mean = points / n;
+    if (dtype == SDFG_F64 || points < (1 << 18) || mean < (1 << 12)) return false;
+    if (steps < 8 && points >= (bf16 ? 5e6 : 12e6)) return false;
+    if (bf16 && points >= 5e6 && mean < (1 << 17)) return false;
+    const double rows = points / (sm_count * 12.0 * 112.0);
+    if (!bf16 && points >= 12e6 && (mean < (1 << 16) || steps < 32)) {
+        c->k = 4;
+        c->seg_rows = rows < 480 ? 96 : rows < 670 ? 160 : 256;
+    } else if (bf16) {
+        c->seg_rows = rows < 25 ? 64 : rows < 50 ? 96 : rows < 300 ? 128 : rows < 590 ? 256 : 384;
+    } else {
+        c->seg_rows = rows < 75 ? 64 : rows < 340 ? 128 : 256;
     }
-    if (bf16 && points / n < (1 << 17)) return false;
-    const int rows = static_cast<int>(points / (152 * 12 * 112) / 3) / 32 * 32;
-    c->seg_rows = std::min(256, std::max(bf16 ? 128 : 96, rows));
-    if (!bf16) c->k = 4;
     return true;
 }
 
@@ -402,16 +415,16 @@ static int plan_build(sdfg_batch_plan **out, const sdfg_desc *desc, int n, int c
         c = *cfg;
     else if (n > 0)
         autotune_lookup(-n, -static_cast<int>(area > 2e9 ? 2e9 : area), dtype, &c);
-    bool scaled_edges = false;
-    if (c.kernel == SDFG_KERNEL_AUTO && c.k == 0 && c.seg_rows == 0 && c.warps == 0) {
-        c.kernel = SDFG_KERNEL_PERSISTENT;
-        if (n > 0 && !any_tol) scaled_edges = untuned_batch(area * n, n, dtype, &c);
-    }
+    const bool untuned = c.kernel == SDFG_KERNEL_AUTO && c.k == 0 && c.seg_rows == 0 && c.warps == 0;
+    if (untuned) c.kernel = SDFG_KERNEL_PERSISTENT;
     if (c.k != 0 && !depth_supported(c.k)) return set_error(SDFG_ERR_INVAL, "batch: k must be 1, 2, 4 or 8");
     if (c.warps < 0 || c.warps > MAX_WARPS || c.seg_rows < 0) return set_error(SDFG_ERR_INVAL, "batch: bad config");
     DeviceState *st = nullptr;
     int rc = current_device(&st);
     if (rc != SDFG_OK) return rc;
+    int steps = 0;
+    for (int g = 0; g < n; ++g) steps = std::max(steps, desc[g].T - desc[g].t_start);
+    const bool scaled_edges = untuned && n > 0 && !any_tol && untuned_batch(area * n, n, steps, dtype, st->sm_count, &c);
 
     sdfg_batch_plan *p = new sdfg_batch_plan();
     p->n = n;
