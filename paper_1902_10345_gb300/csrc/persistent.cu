@@ -33,16 +33,28 @@ __device__ __forceinline__ bool warp_wait(Pred pred, unsigned long long timeout_
     }
 }
 
-template <class ST, int V, bool SE>
+template <class ST, int V, UnitMode M>
 __device__ __forceinline__ bool run_depth(int k, const void *tmap, ST *dst, const GridGeo &g, int s, int q, ST *ring,
                                           uint64_t *bars, uint32_t &ctr, int res, double2 *partial,
-                                          unsigned long long timeout_ns) {
+                                          unsigned long long timeout_ns, bool *large = nullptr) {
     switch (k) {
-        case 1: return run_unit<ST, V, 1, SE>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
-        case 2: return run_unit<ST, V, 2, SE>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
-        case 4: return run_unit<ST, V, 4, SE>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
-        default: return run_unit<ST, V, 8, SE>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns);
+        case 1: return run_unit<ST, V, 1, M>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns, large);
+        case 2: return run_unit<ST, V, 2, M>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns, large);
+        case 4: return run_unit<ST, V, 4, M>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns, large);
+        default: return run_unit<ST, V, 8, M>(tmap, dst, g, s, q, ring, bars, ctr, res, partial, timeout_ns, large);
     }
+}
+// A unit in exact order for the kernel of the scaled grids.  A call, and nothing
+// passed by reference, so that the registers of the scaled units are allocated
+// without it (inlined it spilled 200 bytes there, and the batch of 512 ran 5% slower).
+// Returns the chunk counter, and above it whether the unit ran.
+template <class ST, int V>
+__device__ __noinline__ uint64_t run_exact(int k, const PGrid *G, int srcb, int dstb, int s, int q, ST *ring,
+                                           uint64_t *bars, uint32_t ctr, unsigned long long timeout_ns) {
+    const GridGeo geo = G->geo;
+    const bool ok = run_depth<ST, V, UNIT_EXACT>(k, &G->tm[srcb], static_cast<ST *>(G->buf[dstb]), geo, s, q, ring, bars, ctr,
+                                                 0, nullptr, timeout_ns);
+    return (ok ? 1ull << 32 : 0ull) | ctr;
 }
 
 #ifndef SDFG_PK_MINB
@@ -50,7 +62,11 @@ __device__ __forceinline__ bool run_depth(int k, const void *tmap, ST *dst, cons
 #endif
 
 // SE: fixed-step FP32/BF16 grids only, every unit on the reassociated pipe (see
-// run_unit).
+// run_unit).  A unit that reads a value too large for that pipe (SCALED_LIMIT) in
+// the first pass runs again in exact order, and from the next pass on so do the
+// units around it (no such value gets further in a pass, and none arises, as a step
+// averages); DONE_LARGE in the progress word tells them.  What a unit runs follows
+// from the data alone, not from the order in which units run.
 template <class ST, int V, bool SE>
 __global__ void __launch_bounds__(128, SDFG_PK_MINB) persistent_kernel(const PLaunch L) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -93,6 +109,7 @@ __global__ void __launch_bounds__(128, SDFG_PK_MINB) persistent_kernel(const PLa
                 break;
             }
         }
+        bool large = false;
         if (p > 0) {
             int idx = -1;
             if (lane < 9) {
@@ -100,10 +117,17 @@ __global__ void __launch_bounds__(128, SDFG_PK_MINB) persistent_kernel(const PLa
                 const int q2 = q + lane / 3 - 1;
                 if (s2 >= 0 && s2 < geo.n_strips && q2 >= 0 && q2 < geo.n_segs) idx = unit_off + q2 * geo.n_strips + s2;
             }
-            if (!warp_wait([&] { return idx < 0 || ld_acquire_gpu(L.done + idx) >= p; }, L.timeout_ns)) {
+            int seen = 0;  // this lane's neighbour's progress word
+            auto ready = [&] {
+                if constexpr (!SE) return idx < 0 || ld_acquire_gpu(L.done + idx) >= p;
+                if (idx >= 0) seen = ld_acquire_gpu(L.done + idx);
+                return idx < 0 || (seen & ~DONE_LARGE) >= p;
+            };
+            if (!warp_wait(ready, L.timeout_ns)) {
                 if (lane == 0) set_device_error(L.err, DEV_ERR_TIMEOUT_DEP);
                 break;
             }
+            if (SE) large = __any_sync(FULL_MASK, seen & DONE_LARGE);
         }
         bool skip = false;
         if (G.tol_mode) {
@@ -133,8 +157,23 @@ __global__ void __launch_bounds__(128, SDFG_PK_MINB) persistent_kernel(const PLa
             }
             __syncwarp();
             double2 *partial = res ? L.partials + static_cast<size_t>(cnum & 1) * L.total_units + unit_off + u : nullptr;
-            const bool ok = run_depth<ST, V, SE>(info & PASS_K_MASK, tm, static_cast<ST *>(G.buf[dstb]), geo, s, q, ring,
-                                             bars[warp], ctr, res, partial, L.timeout_ns);
+            const int k = info & PASS_K_MASK;
+            ST *const dst = static_cast<ST *>(G.buf[dstb]);
+            bool ok = true;
+            if constexpr (SE) {
+                if (p == 0)
+                    ok = run_depth<ST, V, UNIT_SCALED_MAX>(k, tm, dst, geo, s, q, ring, bars[warp], ctr, 0, nullptr, L.timeout_ns,
+                                                           &large);
+                else if (!large)
+                    ok = run_depth<ST, V, UNIT_SCALED>(k, tm, dst, geo, s, q, ring, bars[warp], ctr, 0, nullptr, L.timeout_ns);
+                if (ok && large) {
+                    const uint64_t r = run_exact<ST, V>(k, &G, srcb, dstb, s, q, ring, bars[warp], ctr, L.timeout_ns);
+                    ctr = static_cast<uint32_t>(r);
+                    ok = (r >> 32) != 0;
+                }
+            } else {
+                ok = run_depth<ST, V, UNIT_EDGE_EXACT>(k, tm, dst, geo, s, q, ring, bars[warp], ctr, res, partial, L.timeout_ns);
+            }
             if (!ok) {
                 if (lane == 0) set_device_error(L.err, DEV_ERR_TIMEOUT_TMA);
                 break;
@@ -146,7 +185,7 @@ __global__ void __launch_bounds__(128, SDFG_PK_MINB) persistent_kernel(const PLa
         // reader acquires the flag and then fences the async proxy before its
         // TMA loads.
         __syncwarp();
-        if (lane == 0) st_release_gpu(L.done + unit_off + u, p + 1);
+        if (lane == 0) st_release_gpu(L.done + unit_off + u, (SE && large ? DONE_LARGE : 0) | (p + 1));
         if (skip || !res) continue;
 
         // ---- reduce pass: the last unit to finish decides ----

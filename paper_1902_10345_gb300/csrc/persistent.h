@@ -34,6 +34,10 @@ constexpr int PASS_CHECK = 1 << 9;   // a check step: stop if rel <= tol
 constexpr int PASS_FINAL = 1 << 10;  // last step allowed (T cap): always stop, report rel
 constexpr int PASS_REDUCE = PASS_REF | PASS_CHECK | PASS_FINAL;
 
+// In a unit's progress word, beside the passes completed: it ran its last pass
+// in exact order for large values (kernel of the scaled grids).
+constexpr int DONE_LARGE = 1 << 30;
+
 // Buffers of a grid: 0 = caller's out (or its aligned stand-in), 1 = scratch,
 // 2 = caller's in (or its aligned stand-in).
 struct PGrid {  // (aligned as its CUtensorMap members: 128 bytes)
@@ -73,7 +77,7 @@ struct PLaunch {
     const int *n_active;      // [P_max] grids (sorted by P, descending) that have pass p
     const int *units_prefix;  // [n + 1] prefix sums of units over the sorted grids
     const int *order;         // [n] sorted position -> grid index
-    int *done;                // per unit: passes completed
+    int *done;                // per unit: passes completed (and DONE_LARGE)
     double2 *partials;        // [2][total_units] squared-update sums (ref, check)
     int *chk_count;           // per (grid, reduce pass): units finished
     int *head;                // work-queue head

@@ -274,14 +274,21 @@ struct NoHook {
     __device__ __forceinline__ void done(int) {}
 };
 
-// A unit of the persistent kernel's fixed-step variant: it may hold row 0 or
-// row R-1 in the reassociated pipe.
+// A unit of a grid that the persistent kernel holds reassociated throughout: row
+// 0 or row R-1 may be in the reassociated pipe.
 struct EdgeHook : NoHook {
     static constexpr bool EDGES = true;
 };
 
+// Values of this size and larger must not enter the reassociated pipe of a grid
+// that is to be right over the whole range of FP32: its sums grow by 5 a level,
+// 2^18.6 over 8, and an infinity times the negative low half of a scale factor
+// takes its sign.  (2^96 leaves 13 more binary orders below the largest number.)
+constexpr float SCALED_LIMIT = 79228162514264337593543950336.0f;
+
 // CR: rows per TMA chunk (CHUNK_ROWS; the chain kernels stream taller ones).
-template <class ST, int V, int K, bool COLCHK, bool RES, bool EXACT, int CR = CHUNK_ROWS>
+// MAXIN: keep the largest |x| of what is read (step2 only).
+template <class ST, int V, int K, bool COLCHK, bool RES, bool EXACT, int CR = CHUNK_ROWS, bool MAXIN = false>
 struct UnitPipe {
     static_assert(CR % 3 == 0, "chunks are whole turns of the 3-row rotation");
     using CT = typename Store<ST>::CT;
@@ -320,6 +327,7 @@ struct UnitPipe {
     using RT = typename std::conditional<SDFG_RES_FP64 != 0, double, CT>::type;
     RT g_ref, g_chk;
     double acc_ref, acc_chk;
+    float max_in;
     unsigned long long timeout_ns;
 
     __device__ __forceinline__ void issue(int c) {
@@ -482,6 +490,10 @@ struct UnitPipe {
     __device__ __forceinline__ void step2(int r, const ST *src, ST *out) {
         CT x[V];
         VecIO<ST, V>::load(x, src);
+        if constexpr (MAXIN) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) max_in = fmaxf(max_in, fabsf(x[e]));
+        }
 #pragma unroll
         for (int l = 0; l < K; ++l) {
             CT o[V];
@@ -592,6 +604,7 @@ struct UnitPipe {
             g_ref = g_chk = RT(0);
             acc_ref = acc_chk = 0.0;
         }
+        if constexpr (MAXIN) max_in = 0.f;
         int issued = 0;  // chunks whose load was issued
         {
             const int first = n_chunks < STAGES ? n_chunks : STAGES;
@@ -661,16 +674,21 @@ struct UnitPipe {
     }
 };
 
+enum UnitMode {
+    UNIT_EDGE_EXACT,  // units at the ring in exact order, the others reassociated
+    UNIT_SCALED,      // no residuals: reassociated, the ring held scaled and never
+                      // stored (the caller has put it into both grids)
+    UNIT_SCALED_MAX,  // the same; *large: whether it read a value of SCALED_LIMIT or more
+    UNIT_EXACT,       // no residuals: exact order
+};
 // Process unit (strip, seg) of grid `g`: read through tensor map `tmap`
 // (source buffer), write `dst`.  res_flags bit 0: accumulate the squared
 // level-1 update (the first step of a solve), bit 1: the squared level-K
 // update (a check step).  Returns false if a TMA wait ran out.
-// SE (no residuals): the reassociated pipe everywhere, the boundary ring held
-// scaled and never stored (the caller has put it into both grids).
-template <class ST, int V, int K, bool SE = false>
+template <class ST, int V, int K, UnitMode M = UNIT_EDGE_EXACT>
 __device__ __forceinline__ bool run_unit(const void *tmap, ST *dst, const GridGeo &g, int strip, int seg, ST *ring,
                                          uint64_t *bars, uint32_t &chunk_ctr, int res_flags, double2 *partial,
-                                         unsigned long long timeout_ns) {
+                                         unsigned long long timeout_ns, bool *large = nullptr) {
     constexpr int W = 32 * V;
     const int lane = threadIdx.x & 31;
     const int X = strip * g.wout - g.h;
@@ -696,25 +714,30 @@ __device__ __forceinline__ bool run_unit(const void *tmap, ST *dst, const GridGe
 
     bool ok;
     double ar = 0.0, ac = 0.0;
+    constexpr bool SCALED = M == UNIT_SCALED || M == UNIT_SCALED_MAX;
+    constexpr bool MAXIN = M == UNIT_SCALED_MAX;
 #define SDFG_RUN_PIPE(CHK, RS, EX, HOOK)                                                                    \
     {                                                                                                   \
-        UnitPipe<ST, V, K, CHK, RS, EX> p;                                                                  \
+        UnitPipe<ST, V, K, CHK, RS, EX, CHUNK_ROWS, MAXIN> p;                                               \
         p.tmap = tmap; p.dst = dst; p.ld = g.ld; p.R = g.R; p.C = g.C;                                  \
         p.X = X; p.y0 = y0; p.y1 = y1; p.rb = rb; p.n_steps = n_steps; p.n_chunks = n_chunks;           \
-        p.sy0 = SE ? max(y0, 1) : y0; p.sy1 = SE ? min(y1, g.R - 1) : y1;                               \
+        p.sy0 = SCALED ? max(y0, 1) : y0; p.sy1 = SCALED ? min(y1, g.R - 1) : y1;                       \
         p.base = chunk_ctr; p.ring = ring; p.bars = bars; p.lane = lane;                                \
         p.colmask = colmask; p.resmask = resmask; p.own_lane = own_lane; p.full_vec = full_vec;         \
         p.res_flags = res_flags; p.timeout_ns = timeout_ns;                                             \
         HOOK hk;                                                                                        \
         ok = p.run(hk);                                                                                 \
         if (RS) { ar = p.acc_ref; ac = p.acc_chk; }                                                     \
+        if constexpr (MAXIN) *large = __any_sync(FULL_MASK, p.max_in >= SCALED_LIMIT);                  \
     }
     // rows rb .. y1+K-1 are read: a boundary row is among them in the first
     // and the last segments
     const bool rowedge = (rb <= 0) || (y1 + K - 1 >= g.R - 1);
-    if constexpr (SE) {
+    if constexpr (SCALED) {
         if (colchk) SDFG_RUN_PIPE(true, false, false, EdgeHook)
         else SDFG_RUN_PIPE(false, false, false, EdgeHook)
+    } else if constexpr (M == UNIT_EXACT) {
+        SDFG_RUN_PIPE(true, false, true, NoHook)
     } else if (res_flags) {
         if (colchk) SDFG_RUN_PIPE(true, true, true, NoHook)
         else if (rowedge) SDFG_RUN_PIPE(false, true, true, NoHook)
@@ -727,7 +750,7 @@ __device__ __forceinline__ bool run_unit(const void *tmap, ST *dst, const GridGe
 #undef SDFG_RUN_PIPE
     chunk_ctr += static_cast<uint32_t>(n_chunks);
 
-    if (res_flags && partial) {
+    if (M == UNIT_EDGE_EXACT && res_flags && partial) {
         // fixed-order butterfly; lane 0's value is used
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) {
