@@ -14,6 +14,12 @@ namespace sdfg {
 
 constexpr unsigned FULL_MASK = 0xffffffffu;
 
+// Values of this size and larger must not enter unscaled sums of a grid that is to
+// be right over the whole range of FP32: they grow by 5 a step, 2^18.6 over 8,
+// and an infinity times the negative low half of a scale factor takes its sign.
+// (2^96 leaves 13 more binary orders below the largest number.)
+constexpr float SCALED_LIMIT = 79228162514264337593543950336.0f;
+
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

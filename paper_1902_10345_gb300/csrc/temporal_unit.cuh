@@ -280,12 +280,6 @@ struct EdgeHook : NoHook {
     static constexpr bool EDGES = true;
 };
 
-// Values of this size and larger must not enter the reassociated pipe of a grid
-// that is to be right over the whole range of FP32: its sums grow by 5 a level,
-// 2^18.6 over 8, and an infinity times the negative low half of a scale factor
-// takes its sign.  (2^96 leaves 13 more binary orders below the largest number.)
-constexpr float SCALED_LIMIT = 79228162514264337593543950336.0f;
-
 // CR: rows per TMA chunk (CHUNK_ROWS; the chain kernels stream taller ones).
 // MAXIN: keep the largest |x| of what is read (step2 only).
 template <class ST, int V, int K, bool COLCHK, bool RES, bool EXACT, int CR = CHUNK_ROWS, bool MAXIN = false>

@@ -1,4 +1,5 @@
 // Planning and launch of the register-tile kernel (tiles.cuh).
+#include <math.h>
 #include <string.h>
 
 #include <algorithm>
@@ -124,14 +125,20 @@ int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int 
         p.a = static_cast<float>(1.0 - *omega);
         p.b = static_cast<float>(0.25 * *omega);
     }
-    auto split = [](int k, float *hi, float *lo) {
+    for (int last = 0; last < 2; ++last) {
         double f = 1.0;
-        for (int i = 0; i < k; ++i) f = 0.2 * f;
-        *hi = static_cast<float>(f);
-        *lo = static_cast<float>(f - static_cast<double>(*hi));
-    };
-    split(TK_HALO, &p.hi, &p.lo);
-    split(p.k_last, &p.hi_last, &p.lo_last);
+        for (int i = 0; i < (last ? p.k_last : TK_HALO); ++i) f = 0.2 * f;
+        auto split = [](double v, bool down) {
+            TileParams::Factor q;
+            q.hi = static_cast<float>(v);
+            // (rounded down the low half is positive: an infinity keeps its sign)
+            if (down && q.hi > v) q.hi = nextafterf(q.hi, 0.0f);
+            q.lo = static_cast<float>(v - static_cast<double>(q.hi));
+            return q;
+        };
+        p.factor[last] = split(f, false);
+        p.factor_large[last] = split(ldexp(f, TK_DOWN), true);
+    }
     p.timeout_ns = test_hooks().timeout_ns ? test_hooks().timeout_ns : DEFAULT_TIMEOUT_NS;
     // exchange words for two passes, and where a single pass works in place,
     // a grid for the result: a tile may not store what a neighbour still has to load

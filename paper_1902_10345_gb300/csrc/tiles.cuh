@@ -38,7 +38,10 @@
 // is multiplied by 5 each step (as every value is, in effect) and set back to
 // its exact value at the end of a pass.  Points outside the grid may take any
 // value: they reach the interior only through the ring.  BF16 grids stay FP32
-// from load to store.
+// from load to store.  A tile that has loaded or received a value of SCALED_LIMIT or
+// more computes 2^-20 of it from then on (a power of two, which changes no
+// bit of what is not as small as 2^-106), so that no sum overflows which would
+// not in the plain order; no other tile can get one, as a step averages.
 #pragma once
 
 #include <type_traits>
@@ -128,12 +131,16 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
     __shared__ float ring_col[2][BY];      // exact values of columns 0 and C-1 in this box's rows
     __shared__ float ring_row[2][TK_W];    // and of rows 0 and R-1 in its columns
     __shared__ TilePlace place;
+    __shared__ int large;  // the box holds, or has held, a value of SCALED_LIMIT or more (Jacobi)
 
     const int R = P.R, C = P.C;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int warp = tid >> 5;
-    if (tid == 0) place.set(P, TY);
+    if (tid == 0) {
+        place.set(P, TY);
+        large = 0;
+    }
     __syncthreads();
     // (an opaque pointer: see TilePlace)
     auto where = [&]() {
@@ -157,6 +164,19 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
             constexpr int i = decltype(i_t)::value;
             get(X[i], band + i * 32);
         });
+        if constexpr (!SOR) {
+            if (large) {
+                constexpr float DOWN = 1.0f / (1 << TK_DOWN);
+                tk_for<0, RB>([&](auto i_t) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) X[decltype(i_t)::value][e] *= DOWN;
+                });
+            }
+        }
+    };
+    // (every thread that finds one writes the same; read after the next barrier)
+    auto note_large = [&](float m) {
+        if (!SOR && m >= SCALED_LIMIT) large = 1;
     };
 
     // The boundary ring in this box.  Tile row 0 starts at grid row 0 and the
@@ -173,6 +193,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
         const int yb = g.y0 - TK_HALO + warp * RB;  // grid row of the band's first row
         const bool quad_in = gx >= 0 && gx + 4 <= C && P.vec;
         const ST *p = static_cast<const ST *>(P.in) + static_cast<ptrdiff_t>(yb) * P.ld + gx;
+        float m = 0.f;  // (fmaxf passes a NaN over)
 #pragma unroll 6
         for (int i = 0; i < RB; ++i, p += P.ld) {
             float v[4] = {0.f, 0.f, 0.f, 0.f};
@@ -186,7 +207,10 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
                 }
             }
             put(band + i * 32, v);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) m = fmaxf(m, fabsf(v[e]));
         }
+        note_large(m);
         const bool has_l = g.tx == 0, has_r = g.tx == P.nx - 1;
         rq = C - 1 - (g.x0 - TK_HALO);
         er = rq & 3;
@@ -346,7 +370,8 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
         if constexpr (SOR) {
             tk_for<0, RB>([&](auto i_t) { put(band + decltype(i_t)::value * 32, X[decltype(i_t)::value]); });
         } else {
-            const float hi = last ? P.hi_last : P.hi, lo = last ? P.lo_last : P.lo;
+            const TileParams::Factor f = large ? P.factor_large[last] : P.factor[last];
+            const float hi = f.hi, lo = f.lo;
             const float2 h2 = make_float2(hi, hi), l2 = make_float2(lo, lo);
             tk_for<0, RB>([&](auto i_t) {
                 constexpr int i = decltype(i_t)::value;
@@ -440,18 +465,24 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
                 }
                 return ok;
             });
+            float m = 0.f;
 #pragma unroll
             for (int n = 0; n < NR; ++n) {
                 const int h = n * (NT * 2 / TK_W) + hr;
-                if (h < TK_HALO ? ty > 0 : ty + 1 < P.ny)
+                if (h < TK_HALO ? ty > 0 : ty + 1 < P.ny) {
                     *reinterpret_cast<float2 *>(&box[h < TK_HALO ? h : h + BY - 2 * TK_HALO][2 * pr]) = v[n];
+                    m = fmaxf(m, fmaxf(fabsf(v[n].x), fabsf(v[n].y)));
+                }
             }
 #pragma unroll
             for (int n = 0; n < NC; ++n) {
                 const int r = n * (NT / TK_HALO) + (tid >> 3);
-                if (side_ok && r < TY)
+                if (side_ok && r < TY) {
                     *reinterpret_cast<float2 *>(&box[TK_HALO + r][(sd ? TK_W - TK_HALO : 0) + (tid & 3) * 2]) = v[NR + n];
+                    m = fmaxf(m, fmaxf(fabsf(v[NR + n].x), fabsf(v[NR + n].y)));
+                }
             }
+            note_large(m);
         }
         __syncthreads();
         take_band();

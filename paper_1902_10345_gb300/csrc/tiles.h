@@ -7,6 +7,7 @@
 
 namespace sdfg {
 
+constexpr int TK_DOWN = 20;                       // binary orders a tile with large values is scaled down by
 constexpr int TK_HALO = 8;                        // halo rows and columns = steps per pass
 constexpr int TK_W = 128;                         // box columns, 4 per lane
 constexpr int TK_TX = TK_W - 2 * TK_HALO;         // 112 columns per tile
@@ -21,7 +22,11 @@ struct TileParams {
     int nx, ny;       // tiles
     int vec;          // rows can be read and written four columns at a time
     int n_pass, k_last;  // passes, steps (SOR: half-sweeps) of the last one
-    float hi, lo, hi_last, lo_last;  // 0.2^8 and 0.2^k_last as hi + lo
+    // the factor at the end of a pass as hi + lo: 0.2^8 and 0.2^k_last, and the
+    // same times 2^TK_DOWN for tiles with large values
+    struct Factor {
+        float hi, lo;
+    } factor[2], factor_large[2];
     float a, b;       // SOR: 1 - omega, omega / 4
     unsigned long long timeout_ns;
 };
