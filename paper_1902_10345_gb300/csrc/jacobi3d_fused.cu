@@ -18,9 +18,14 @@
 // per plane.
 //
 // Arithmetic as in the 2-D units (level_p in temporal_unit.cuh): sums carried
-// unscaled (level l holds 7^l times the state), 7^-K applied once as hi + lo.
-// The fixed shell is held scaled like every other value (times 7 at each
-// level) and never stored: j3_shell_copy puts it into both ping-pong boxes.
+// unscaled, 7^-K applied once as hi + lo.  So that nothing overflows that does not
+// in the plain order, level 0 makes its sums 8^-(K-1) of what they are (a power of
+// two, inside multiply-adds: 2 products more per 4 points): level l > 0 holds 7^l
+// 8^(1-K) times the state, at most 7 times at the end, and loses no bit of values
+// above 2^-117.  hi is rounded down, which makes lo positive: an infinity times
+// either keeps its sign.  The fixed shell is held scaled like every other value
+// (times 7 at each level) and never stored: j3_shell_copy puts it into both
+// ping-pong boxes.
 //
 // What bounds it: one step per launch is bound by HBM (8 bytes per FP32 update:
 // 512^3 at 172 us per step, 0.9 of the measured bandwidth).  Here it is issue:
@@ -29,6 +34,7 @@
 // tiles past the grid's end, 2K planes per run along z); DRAM is at 30%.
 // Measured on 512^3, us per step, warps x rows: K=2 16x3 107, 12x5 106; K=3
 // 12x3 100, 8x5 117, 16x2 125, 12x4 and 8x6 spill (115, 122); K=4 8x4 113.
+#include <math.h>
 #include <string.h>
 
 #include <algorithm>
@@ -66,6 +72,7 @@ __global__ void __launch_bounds__(32 * NW, 1) jacobi3d_fused_kernel(const __grid
     constexpr int XH = 16 / sizeof(ST);  // column halo: 16 bytes, so the box start stays TMA-aligned
     constexpr int TX = W - 2 * XH;
     static_assert(XH >= K && TY > 0 && BY <= 256, "halo");
+    constexpr float DOWN = 1.0f / (1 << 3 * (K - 1));  // of level 0's sums
     constexpr uint32_t PLANE_BYTES = BY * W * sizeof(ST);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bars[JF_NS];
@@ -164,20 +171,26 @@ __global__ void __launch_bounds__(32 * NW, 1) jacobi3d_fused_kernel(const __grid
             jf_for<0, RB>([&](auto i_t) {
                 constexpr int i = decltype(i_t)::value;
                 const float(&a)[4] = A[Q ^ 1][l][i];
+                constexpr float SEVEN = l == 0 ? 7.0f * DOWN : 7.0f;
                 float o[4];
-                jf_add(o, P[l][i], A[Q][l][i]);
+                if constexpr (l == 0) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) o[e] = __fmaf_rn(A[Q][l][i][e], DOWN, P[l][i][e]);
+                } else {
+                    jf_add(o, P[l][i], A[Q][l][i]);
+                }
                 if constexpr (VAR == 1) {
-                    if (lane_l) o[0] = __fmul_rn(7.0f, a[0]);
+                    if (lane_l) o[0] = __fmul_rn(SEVEN, a[0]);
                 }
                 if constexpr (VAR >= 4) {
-                    if (lane_r) o[VAR - 4] = __fmul_rn(7.0f, a[VAR - 4]);
+                    if (lane_r) o[VAR - 4] = __fmul_rn(SEVEN, a[VAR - 4]);
                 }
                 if constexpr (VAR == 2 || VAR == 3) {
                     const int zc = zi - l - 1, r = yb + i;  // the plane this level finishes
                     const unsigned m4 = VAR == 3 && (zc <= 0 || zc >= g.D - 1 || r <= 0 || r >= g.R - 1) ? 15u : colmask;
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
-                        if ((m4 >> e) & 1u) o[e] = __fmul_rn(7.0f, a[e]);
+                        if ((m4 >> e) & 1u) o[e] = __fmul_rn(SEVEN, a[e]);
                 }
                 if constexpr (l + 1 < K) {
 #pragma unroll
@@ -225,8 +238,11 @@ __global__ void __launch_bounds__(32 * NW, 1) jacobi3d_fused_kernel(const __grid
                 constexpr int i = decltype(i_t)::value;
                 const float left = __shfl_up_sync(FULL_MASK, x[i][3], 1);
                 const float right = __shfl_down_sync(FULL_MASK, x[i][0], 1);
-                const float q0 = __fadd_rn(x[i][0], x[i][1]), q1 = __fadd_rn(x[i][2], x[i][3]);
-                const float h[4] = {__fadd_rn(left, q0), __fadd_rn(q0, x[i][2]), __fadd_rn(x[i][1], q1), __fadd_rn(q1, right)};
+                // (x + y, level 0: x DOWN + y, with y scaled already)
+                auto plus = [](float u, float v) { return l == 0 ? __fmaf_rn(u, DOWN, v) : __fadd_rn(u, v); };
+                float q0 = __fadd_rn(x[i][0], x[i][1]), q1 = __fadd_rn(x[i][2], x[i][3]);
+                if constexpr (l == 0) q0 = __fmul_rn(q0, DOWN), q1 = __fmul_rn(q1, DOWN);
+                const float h[4] = {plus(left, q0), plus(x[i][2], q0), plus(x[i][1], q1), plus(right, q1)};
                 float t[4];
                 float n[4], s[4];
 #pragma unroll
@@ -236,7 +252,8 @@ __global__ void __launch_bounds__(32 * NW, 1) jacobi3d_fused_kernel(const __grid
                 }
                 jf_add(t, n, s);
                 jf_add(t, t, A[Q ^ 1][l][i]);
-                jf_add(P[l][i], t, h);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) P[l][i][e] = plus(t[e], h[e]);
             });
         });
         out += g.plane;
@@ -374,9 +391,11 @@ int launch_j3_fused(const CUtensorMap &tm, void *dst, const J3FGeo &g, int K, in
     const size_t smem = static_cast<size_t>(JF_NS) * j3_fused_rows(K) * 128 * dtype_bytes(dtype);
     int rc = raise_smem_limit(fn, smem);
     if (rc != SDFG_OK) return rc;
-    double f = 1.0;
+    double f = ldexp(1.0, 3 * (K - 1));
     for (int i = 0; i < K; ++i) f /= 7.0;
-    float hi = static_cast<float>(f), lo = static_cast<float>(f - static_cast<double>(hi));
+    float hi = static_cast<float>(f);
+    if (hi > f) hi = nextafterf(hi, 0.0f);
+    float lo = static_cast<float>(f - static_cast<double>(hi));
     CUtensorMap t = tm;
     J3FGeo gg = g;
     void *dp = dst;

@@ -134,3 +134,46 @@ def test_tiles(shape, T, dtype, what):
     binding.jacobi2d(x, y, T)
     compare(y, jacobi2d64(x, T), put, T, 1 if dtype == torch.bfloat16 else 0)
     assert binding.sdfg_device_error(True) == 0
+
+
+def jacobi3d64(x, T):
+    a = x.double()
+    c = a[1:-1, 1:-1, 1:-1]
+    for _ in range(T):
+        s = (a[1:-1, :-2, 1:-1] + a[1:-1, 2:, 1:-1]) + (a[1:-1, 1:-1, :-2] + a[1:-1, 1:-1, 2:])
+        c.copy_((c + (s + (a[:-2, 1:-1, 1:-1] + a[2:, 1:-1, 1:-1]))) / 7.0)
+    return a
+
+
+@pytest.mark.parametrize("what", ["shell inf", "point -inf", "inf and -inf", "nan", "shell large", "point large", "all large"])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("T", [1, 2, 3, 4, 7])
+def test_box(T, dtype, what):
+    """The 7-point stencil: one step, passes of 2 and of 3; 3.5e37, seven of which add up to an FP32 number."""
+    torch.manual_seed(6)
+    D, R, C = 21, 70, 263
+    x = torch.rand((D, R, C + 1), device="cuda").to(dtype)[:, :, :C]
+    put = torch.zeros(x.shape, dtype=torch.bool, device="cuda")
+    every = (slice(None),) * 3
+    for at, v in {
+        "shell inf": [((0, slice(None), slice(None)), INF)],
+        "point -inf": [((9, 33, 130), -INF)],
+        "inf and -inf": [((slice(None), 0, slice(None)), INF), ((slice(None), slice(None), C - 1), -INF), ((5, 5, 5), INF)],
+        "nan": [((11, 20, 121), NAN)],
+        "shell large": [((D - 1, slice(None), slice(None)), 3.5e37), ((slice(None), slice(None), 0), -3.5e37)],
+        "point large": [((9, 33, 119), 3.5e37)],
+        "all large": [(every, 3.5e37)],
+    }[what]:
+        x[at] = v
+        put[at] = True
+    y = torch.empty_strided(x.shape, x.stride(), dtype=dtype, device="cuda")
+    binding.jacobi3d(x, y, T)
+    got, want = y.double(), jacobi3d64(x, T)
+    assert torch.equal(got.isnan(), want.isnan())
+    assert torch.equal(got.isinf(), want.isinf()) and torch.equal(got[got.isinf()], want[want.isinf()])
+    # seven roundings a step and the pass's factors; BF16 one per pass or step
+    rel = 12 * T * 2.0 ** -24 + (T * 2.0 ** -8 if dtype == torch.bfloat16 else 0.0)
+    fin = want.isfinite()
+    err = torch.where(fin, (got - want).abs(), 0.0)
+    assert float(err.max()) <= rel * max(1.0, float(torch.where(fin, want.abs(), 0.0).max()))
+    assert binding.sdfg_device_error(True) == 0
