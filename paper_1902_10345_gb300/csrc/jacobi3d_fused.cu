@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(32 * NW, 1) jacobi3d_fused_kernel(const __grid
     constexpr int XH = 16 / sizeof(ST);  // column halo: 16 bytes, so the box start stays TMA-aligned
     constexpr int TX = W - 2 * XH;
     static_assert(XH >= K && TY > 0 && BY <= 256, "halo");
+    static_assert(RB <= 3, "(RB - 1) ld fits 32 unsigned bits");
     constexpr float DOWN = 1.0f / (1 << 3 * (K - 1));  // of level 0's sums
     constexpr uint32_t PLANE_BYTES = BY * W * sizeof(ST);
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -200,7 +201,8 @@ __global__ void __launch_bounds__(32 * NW, 1) jacobi3d_fused_kernel(const __grid
                     const float2 f = __ffma2_rn(u, make_float2(hi, hi), __fmul2_rn(u, make_float2(lo, lo)));
                     const float2 h2 = __ffma2_rn(v, make_float2(hi, hi), __fmul2_rn(v, make_float2(lo, lo)));
                     const float w[4] = {f.x, f.y, h2.x, h2.y};
-                    ST *p = out + i * g.ld;
+                    // (a row of the band is at most two pitches off: 32 unsigned bits hold that)
+                    ST *p = out + static_cast<unsigned>(i) * static_cast<unsigned>(g.ld);
                     const int pred = rows & (1u << i);
                     if constexpr (VAR == 0) {
                         store_pred(p, w, pred);
