@@ -332,8 +332,8 @@ int sdfg_laplace1d(double *A, int N, int T, void *stream);
  *   (1/7) * (c + (((n + s) + (w + e)) + (u + d)))
  * (n, s: rows i-1, i+1; w, e: columns j-1, j+1; u, d: planes z-1, z+1), in
  * that order, round to nearest, in FP64 for FP64 (bit-identical to a plain FP64
- * loop).  FP32 and BF16 storage compute in FP32 and, from T = 2 on, fuse two or
- * three steps per pass: sums carried unscaled in another order and scaled once
+ * loop).  FP32 and BF16 storage compute in FP32 and, from T = 2 on (a box of at
+ * most 8 planes of 786432 points or more apart), fuse two or three steps per pass: sums carried unscaled in another order and scaled once
  * per pass, which is more accurate against FP64; BF16 is rounded when a pass
  * stores the box.  The one-cell outer shell keeps its input values.  out receives the
  * whole box after T steps; in is read only; in == out is allowed; T = 0, or

@@ -11,8 +11,8 @@
 //
 // Passes: FP32 and BF16 boxes advance 3 steps per launch, and 2 where T is no
 // multiple of 3 (jacobi3d_fused.cu; 512^3 T=100 17.5 -> 10.3 ms, a seventh of
-// the error); a single step runs on jacobi3d_kernel, FP64 on
-// jacobi3d_flat_kernel.
+// the error); a single step, and every step of a box of few large planes, runs on
+// jacobi3d_kernel, FP64 on jacobi3d_flat_kernel.
 //
 // jacobi3d_kernel: one launch is one timestep.  A CTA owns a tile of TY rows x TX columns and
 // streams through a range of planes (2.5-D blocking, paper App. B MapTiling
@@ -345,10 +345,14 @@ extern "C" int sdfg_jacobi3d(const void *in, void *out, int depth, int rows, int
     }
     const size_t S = dtype_bytes(dtype);
     // FP32 and BF16 storage: passes of 3 fused steps, and of 2 where T is no
-    // multiple of 3; a single step runs alone
+    // multiple of 3; a single step runs alone, and so do all of them on a box of at
+    // most 8 large planes, whose halo planes are most of a pass.  us, one at a time and
+    // fused, T=9, FP32: 3 x 1200 x 1200 77, 111; 8 x 1000 x 1000 128, 151; 8 x 1200 x
+    // 1200 152, 160; 10 x 1200 x 1200 174, 173; 3 x 600 x 600 58, 46; 8 x 600 x 600 94, 67
     const bool f64 = dtype == SDFG_F64;
+    const bool fused = !f64 && T > 1 && (depth > 8 || static_cast<long long>(rows) * cols < (3 << 18));
     int n_two = 0, n_pass = T;
-    if (!f64 && T > 1) {
+    if (fused) {
         n_two = (3 - T % 3) % 3;
         n_pass = n_two + (T - 2 * n_two) / 3;
     }
@@ -405,10 +409,13 @@ extern "C" int sdfg_jacobi3d(const void *in, void *out, int depth, int rows, int
             rc = launch_j3_flat(fin, dst, g, st->sm_count, s);
             done();
         }
-    } else if (T == 1) {
+    } else if (!fused) {
         encode(j3_box_cols(dtype), J3_BY);
-        if (rc == SDFG_OK) rc = launch_j3(tm[0], dst, plan_j3(depth, rows, cols, ldw, dtype, st->sm_count), dtype, st->d_err, s);
-        done();
+        const J3Geo g = plan_j3(depth, rows, cols, ldw, dtype, st->sm_count);
+        for (int t = 0; t < T && rc == SDFG_OK; ++t) {
+            rc = launch_j3(src_map(), dst, g, dtype, st->d_err, s);
+            done();
+        }
     } else {
         // the fused kernel stores interior points only
         rc = j3_shell_copy(src0, first, second == src0 || n_pass == 1 ? nullptr : second, depth, rows, cols, ldw, dtype, s);
