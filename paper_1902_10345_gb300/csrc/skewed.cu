@@ -298,18 +298,27 @@ int chain_plan_build(ChainPlan *c, DeviceState *st, cudaStream_t s) {
 // warp; on a large one the passes in flight hide it.  GUpdates/s at T=160,
 // 640-row chains publishing every 8 chunks -> this: FP32 2400^2 765 -> 1707,
 // 3000^2 1129 -> 2330, 4096^2 1979 -> 3599, 5600^2 3343 -> 4701, 7000^2 4614 ->
-// 5120, 8192^2 as before.  BF16 (512 rows, 6 chunks before) 2400^2 767 -> 1184,
-// 3000^2 1106 -> 1571, 4096^2 1817 -> 2319, 5600^2 2910 -> 3407, 7000^2 3727 ->
-// 4186; its warps hold two thirds more rows per chunk, so long chains that
-// publish every chunk beat short ones.
-static void chain_defaults(long long points, int dtype, int *L, int *pub) {
+// 5120, 8192^2 as before.
+// BF16 holds two thirds more rows per chunk, so over many passes long chains that
+// publish every chunk beat short ones; with few passes in flight, and in the
+// shallower passes of the remainder, it is the number of chains that counts, as in
+// FP32.  us, 512 rows publishing every 6 chunks, and every chunk at 512, 128 rows: T=8
+// 3000^2 149, 159, 68; 6000^2 183, 195, 117; T=160 3000^2 1300, 865, 968; 6000^2 1849,
+// 1467, 1755; T=159 (three passes more) 3000^2 -, 1161, 1116; 6000^2 -, 1874, 1887.  They
+// meet at T = 140, 96, 70, 55, 50, 40 on 2400^2, 3000^2, 4096^2, 5000^2, 6000^2, 7000^2,
+// and about 32 steps later for each pass of the remainder.
+static void chain_defaults(long long points, long long T, int k, int dtype, int *L, int *pub) {
     int l = 640, p = chain_pub_chunks(dtype_bytes(dtype));
     if (dtype == SDFG_F32 && points < (58LL << 20)) {
         l = 128;
         p = points < (24LL << 20) ? 1 : points < (40LL << 20) ? 2 : 8;
     } else if (dtype == SDFG_BF16) {
-        l = points < (8LL << 20) ? 256 : points < (58LL << 20) ? 640 : 512;
-        if (points < (58LL << 20)) p = 1;
+        l = 512;
+        if (points < (58LL << 20)) {
+            const int rest = static_cast<int>(plan_passes(T % k, k).size());
+            if (static_cast<double>(T) < 30.0 + 6e8 / static_cast<double>(points) + 32.0 * rest) l = 128;
+            p = 1;
+        }
     }
     if (*pub <= 0) *pub = *L <= 0 ? p : chain_pub_chunks(dtype_bytes(dtype));
     if (*L <= 0) *L = l;
@@ -321,7 +330,7 @@ static void chain_defaults(long long points, int dtype, int *L, int *pub) {
 // TMA-compatible.
 int run_single_chain(const void *in, void *out, int R, int C, int ld, long long T, int dtype, int k, int L, int pub,
                      DeviceState *st, cudaStream_t s) {
-    chain_defaults(static_cast<long long>(R) * C, dtype, &L, &pub);
+    chain_defaults(static_cast<long long>(R) * C, T, k, dtype, &L, &pub);
     L = std::max(L, 4 * k);
     std::lock_guard<std::mutex> lk(g_chain_mu);
     ChainPlan *c = nullptr;
