@@ -65,8 +65,10 @@
  *
  * Errors: every function returns an sdfg_status.  Argument errors are found
  * on the host before any work is enqueued.  Errors of the CUDA runtime are
- * returned as SDFG_ERR_CUDA.  A device-side wait that runs out (persistent
- * kernels) records SDFG_ERR_TIMEOUT in a per-device error word, which
+ * returned as SDFG_ERR_CUDA.  A device-side wait that runs out (for the rows of
+ * another unit, chain or tile, or for a TMA load) records SDFG_ERR_TIMEOUT in a
+ * per-device error word; an asynchronous call has returned by then, and what it
+ * wrote is no result.  The word is what
  * sdfg_device_error() reads.  sdfg_last_error() returns a thread-local
  * message about the most recent failure on the calling thread.
  */
@@ -409,10 +411,11 @@ const char *sdfg_last_error(void);
 /*
  * Test hooks for the failure paths (no GPU fault is involved):
  *   hook 1, value 0/1: persistent launches created afterwards make their first
- *           work item wait on a flag that nothing sets, so the bounded wait
+ *           work item wait on a flag that nothing sets, and tile launches their
+ *           halos wait for a pass that never comes, so the bounded wait
  *           runs out and the launch reports SDFG_ERR_TIMEOUT;
- *   hook 2, value ns: limit of every bounded device wait in persistent
- *           launches created afterwards (0 = default, 2 s);
+ *   hook 2, value ns: limit of every bounded device wait in persistent and
+ *           tile launches created afterwards (0 = default, 2 s);
  *   hook 3, value n: batch plans created afterwards with SDFG_KERNEL_SKEWED
  *           put fixed-step grids of at least n points on chains (-1 =
  *           default, 2^20; 0 = every fixed-step grid);

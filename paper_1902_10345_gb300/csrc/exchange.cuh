@@ -6,10 +6,13 @@
 
 namespace sdfg {
 
+constexpr uint32_t LL_NEVER = 1u << 31;  // added to a pass's number: one that no launch reaches
+
 // Exchange words: a value and the number of the pass it belongs to in one
 // 64-bit word, two words per 16-byte access.  A word arrives whole, so the
 // reader needs no flag and no fence: it reads until every word bears the pass
-// it waits for.
+// it waits for.  (Data and flag in one word is the idea of the low-latency
+// protocol, LL, of NVIDIA's NCCL, whose public documents describe it.)
 __device__ __forceinline__ void ll_store(uint64_t *p, float x, float y, uint32_t pass) {
     asm volatile(
         "{\n\t.reg .b64 a, b;\n\t"

@@ -142,6 +142,7 @@ int run_tiles(const void *in, void *out, int R, int C, int ld, long long T, int 
         p.factor_large[last] = split(ldexp(f, TK_DOWN), true);
     }
     p.timeout_ns = test_hooks().timeout_ns ? test_hooks().timeout_ns : DEFAULT_TIMEOUT_NS;
+    p.stuck = test_hooks().inject_stuck_wait ? LL_NEVER : 0;
     // exchange words for two passes, and where a single pass works in place,
     // a grid for the result: a tile may not store what a neighbour still has to load
     const bool staged = in == out && p.n_pass == 1;

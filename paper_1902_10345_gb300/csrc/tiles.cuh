@@ -436,6 +436,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
             const uint64_t *const cols =
                 xc + (static_cast<ptrdiff_t>((sd ? tx + 1 : tx - 1) * 2 + 1 - sd) * R + g.y0) * TK_HALO + (tid & 3) * 2;
             float2 v[NR + NC];
+            const uint32_t expect = stamp + P.stuck;
             // (every thread loads every time, what lies off the grid from the
             // first word and unchecked: loads under conditions would wait for
             // one another)
@@ -444,7 +445,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
             wait.until([&]() -> bool {
                 const bool want = col_ok && ty > 0;
                 const int r = tid >> 3;
-                return ll_load(v[0].x, v[0].y, want ? rows + static_cast<ptrdiff_t>(hr) * P.ldx : side_ok && r < TY ? cols + r * TK_HALO : xr, stamp) ||
+                return ll_load(v[0].x, v[0].y, want ? rows + static_cast<ptrdiff_t>(hr) * P.ldx : side_ok && r < TY ? cols + r * TK_HALO : xr, expect) ||
                        !(want || (side_ok && r < TY));
             });
             wait.until([&]() -> bool {
@@ -455,13 +456,13 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) tile_kernel(const __grid_con
                     const bool want = col_ok && (h < TK_HALO ? ty > 0 : ty + 1 < P.ny);
                     // (above: the "down" rows of tile row ty-1; below: the "up" rows of ty+1)
                     const uint64_t *const p = rows + static_cast<ptrdiff_t>(h < TK_HALO ? h : h + 2 * TK_HALO) * P.ldx;
-                    ok &= ll_load(v[n].x, v[n].y, want ? p : xr, stamp) || !want;
+                    ok &= ll_load(v[n].x, v[n].y, want ? p : xr, expect) || !want;
                 }
 #pragma unroll
                 for (int n = 0; n < NC; ++n) {
                     const int r = n * (NT / TK_HALO) + (tid >> 3);
                     const bool want = side_ok && r < TY;
-                    ok &= ll_load(v[NR + n].x, v[NR + n].y, want ? cols + r * TK_HALO : xr, stamp) || !want;
+                    ok &= ll_load(v[NR + n].x, v[NR + n].y, want ? cols + r * TK_HALO : xr, expect) || !want;
                 }
                 return ok;
             });

@@ -29,6 +29,7 @@ struct TileParams {
     } factor[2], factor_large[2];
     float a, b;       // SOR: 1 - omega, omega / 4
     unsigned long long timeout_ns;
+    unsigned stuck;  // test hook: the halo waits are for passes that far ahead (0: none)
 };
 
 // First column and row of a tile: the first tile starts at 0, the last ends at

@@ -43,6 +43,7 @@ struct Tile64Params {
     int box;          // elements of the box
     int n_pass, k_last;
     unsigned long long timeout_ns;
+    unsigned stuck;   // test hook: the halo waits are for passes that far ahead (0: none)
 };
 
 __global__ void __launch_bounds__(T64_THREADS, 1) tile64_kernel(const __grid_constant__ Tile64Params P) {
@@ -128,7 +129,7 @@ __global__ void __launch_bounds__(T64_THREADS, 1) tile64_kernel(const __grid_con
             wait.until([&]() -> bool {
                 bool ok = true;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) ok &= ll_load(v[q], src[q], stamp) || to[q] < 0;
+                for (int q = 0; q < 4; ++q) ok &= ll_load(v[q], src[q], stamp + P.stuck) || to[q] < 0;
                 return ok;
             });
 #pragma unroll
@@ -192,6 +193,7 @@ int run_tiles64(const void *in, void *out, int R, int C, int ld, long long T, De
     p.n_pass = static_cast<int>((T + p.K - 1) / p.K);
     p.k_last = static_cast<int>(T - static_cast<long long>(p.n_pass - 1) * p.K);
     p.timeout_ns = test_hooks().timeout_ns ? test_hooks().timeout_ns : DEFAULT_TIMEOUT_NS;
+    p.stuck = test_hooks().inject_stuck_wait ? LL_NEVER : 0;
     const size_t smem = 2 * sizeof(double) * static_cast<size_t>(p.box);
     const void *fn = reinterpret_cast<const void *>(&tile64_kernel);
     SDFG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
