@@ -42,6 +42,12 @@
 // more computes 2^-20 of it from then on (a power of two, which changes no
 // bit of what is not as small as 2^-106), so that no sum overflows which would
 // not in the plain order; no other tile can get one, as a step averages.
+// (The test of what each exchange brings and of the flag is some 20 instructions a
+// pass, which cost nothing measurable on the tallest tiles, 2048^2 T=1024 1348 -> 1331 us,
+// and up to 5% of FP32 and 9% of BF16 passes on grids of 400^2 to 1000^2, 1000^2 T=300 180 ->
+// 189 and 176 -> 188 us.  A kernel in the memset's place that looks the grid over first
+// spares those and costs the tall ones 4%; an agreement between the tiles during the
+// first pass cost as much as the test.)
 #pragma once
 
 #include <type_traits>

@@ -130,9 +130,20 @@ def test_tiles(shape, T, dtype, what):
     torch.manual_seed(5)
     x.copy_(torch.rand(shape, device="cuda"))
     put = plant(x, what)
+    if what in ("point inf", "point large"):
+        x[-1, :] = 1e-38  # the ring is copied exactly
     y = torch.empty_strided(x.shape, x.stride(), dtype=dtype, device="cuda")
     binding.jacobi2d(x, y, T)
-    compare(y, jacobi2d64(x, T), put, T, 1 if dtype == torch.bfloat16 else 0)
+    want = jacobi2d64(x, T)
+    compare(y, want, put, T, 1 if dtype == torch.bfloat16 else 0)
+    for got, was in ((y[0], x[0]), (y[-1], x[-1]), (y[:, 0], x[:, 0]), (y[:, -1], x[:, -1])):
+        assert torch.equal(got.nan_to_num(7.0), was.nan_to_num(7.0))
+    if what == "nan":
+        x.nan_to_num_(0.25)
+        x[3, 3] = BIG
+        binding.jacobi2d(x, y, T)
+    binding.jacobi2d(x, x, T)  # in place: the same
+    assert torch.equal(x.nan_to_num(7.0), y.nan_to_num(7.0))
     assert binding.sdfg_device_error(True) == 0
 
 
