@@ -67,6 +67,7 @@ def parse():
     p.add_argument("--precision-grids", type=int, default=4, help="precision: 16384^2 grids per storage type")
     p.add_argument("--batch-grids", type=int, default=512,
                    help="batch: grids in the batch (the first n of the seeded 512; smaller batches for profiling)")
+    p.add_argument("--untuned", action="store_true", help="batch: the library's own choice, without the autotuner")
     p.add_argument("--line-requests", type=int, default=1000,
                    help="default line: served requests (a prefix of the seeded 10,000-request trace)")
     p.add_argument("--line-plain-seconds", type=float, default=90.0,
@@ -536,8 +537,8 @@ def _padded(R, C, dtype, device="cuda"):
 def measure_batch(a, steps: int, warmup: int, n_grids: int = 512):
     """512 uneven grids (rows, cols log-uniform in [64, 2048], T in [50, 500])
     in ONE persistent launch, replayed through a captured CUDA graph; k and
-    the segment height from the project's batch autotuner unless --k or
-    --seg-rows fix them.  n_grids < 512 takes the first n_grids of the same
+    the segment height from the project's batch autotuner (which may choose the
+    library's own way of running the batch) unless --k or --seg-rows fix them.  n_grids < 512 takes the first n_grids of the same
     seeded batch (for profiling).  Returns the block of the JSON line."""
     import ctypes
 
@@ -563,6 +564,8 @@ def measure_batch(a, steps: int, warmup: int, n_grids: int = 512):
                                                 else "persistent"),
                              k=a.k or 8, seg_rows=a.seg_rows or 96, warps=a.warps or 4)
         tuned = False
+    elif a.untuned:
+        cfg, tuned = binding.config(), False
     else:
         # the project's autotuner picks k and the segment height on this batch
         cfg = binding.sdfg_autotune_batch(descs, 64)
@@ -587,7 +590,9 @@ def measure_batch(a, steps: int, warmup: int, n_grids: int = 512):
     binding.check(L.sdfg_batch_plan_destroy(plan))
     assert all(d.status == 0 and d.steps_done == sp.T for d, sp in zip(arr, specs))
     value = updates * steps / (ms / 1e3) / 1e9
-    k = cfg.k
+    # the library's own choice for this batch (kernel 0): depth 8, 256-row segments
+    own = cfg.kernel == binding.SDFG_KERNEL_AUTO
+    k, seg_rows = (8, 256) if own else (cfg.k, cfg.seg_rows)
     # passes of the plan: plan_passes(T, k) = T // k passes of k, then the remainder in powers of two
     def n_passes(T):
         return T // k + bin(T % k).count("1")
@@ -596,12 +601,13 @@ def measure_batch(a, steps: int, warmup: int, n_grids: int = 512):
     hbm, src = measured_peaks()
     achieved = bytes_per_step / (ms / steps / 1e3) / 1e9
     persistent = cfg.kernel != binding.SDFG_KERNEL_SKEWED
-    traffic = committed_traffic(build.kernel_digest(None), wl) if persistent else None
+    traffic = committed_traffic(build.kernel_digest(None), wl if own else f"{wl}_k{k}_seg{seg_rows}") if persistent else None
     # kernels one replay launches (no grid of this batch solves to a tolerance,
-    # so no finalize launch): the persistent kernel; or the ring copy and the
+    # so no finalize launch): the persistent kernel (the library's own choice: and
+    # the ring copy before it); or the ring copy and the
     # chain kernel, plus the persistent kernel for grids under 2^20 points
     if persistent:
-        per_step = 1
+        per_step = 2 if own else 1
     else:
         per_step = 2 + (1 if any(sp.rows * sp.cols < (1 << 20) for sp in specs) else 0)
     del xs, ys
@@ -610,8 +616,9 @@ def measure_batch(a, steps: int, warmup: int, n_grids: int = 512):
         "value": value, "unit": UNIT, "steps": steps, "warmup": max(3, warmup), "ms_per_step": ms / steps,
         "launches_per_step": per_step,
         "config": {"workload": wl, "grids": n_grids, "updates_per_step": updates,
-                   "k": k, "seg_rows": cfg.seg_rows, "autotuned": tuned, "passes_per_step": passes,
+                   "k": k, "seg_rows": seg_rows, "autotuned": tuned, "passes_per_step": passes,
                    "kernel": ("chain kernel" if cfg.kernel == binding.SDFG_KERNEL_SKEWED else "persistent kernel")
+                             + (", every unit reassociated" if own else "")
                              + " (one launch per step, replayed from a captured CUDA graph)",
                    "layout": "each grid pitched to a multiple of 4 columns (16-byte rows)",
                    "l2": "1.3 GB resident, larger than L2, no flush" if n_grids == 512 else "first grids of the batch"},

@@ -339,9 +339,10 @@ int sdfg_laplace1d(double *A, int N, int T, void *stream);
  * per pass, which is more accurate against FP64; BF16 is rounded when a pass
  * stores the box.  The one-cell outer shell keeps its input values.  out receives the
  * whole box after T steps; in is read only; in == out is allowed; T = 0, or
- * an extent below 3, copies.  in/out should be 16-byte aligned with ld *
- * sizeof(element) a multiple of 16; otherwise the box is staged through an
- * aligned copy.  Scratch: one box (two when staged), stream-ordered.
+ * an extent below 3, copies.  FP32 and BF16: in/out should be 16-byte aligned
+ * with ld * sizeof(element) a multiple of 16; otherwise the box is staged through
+ * an aligned copy (FP64 takes any layout).  Scratch: one box (two when staged),
+ * stream-ordered.
  * Asynchronous on `stream`.  SDFG_ERR_INVAL for negative extents or T, ld <
  * cols, an unknown dtype or a null pointer with a non-empty box.
  */

@@ -30,8 +30,9 @@
 // What bounds it: one step per launch is bound by HBM (8 bytes per FP32 update:
 // 512^3 at 172 us per step, 0.9 of the measured bandwidth).  Here it is issue:
 // about 40 instructions per 4 points and level, of which 24 are the arithmetic,
-// at 59% of the issue slots, on 1.6 times the points (halo rows and columns,
-// tiles past the grid's end, 2K planes per run along z); DRAM is at 30%.
+// at 59% of the issue slots, on 1.75 times the points (in the plane 1.59: 5 tile
+// columns of 128 lanes and 18 tile rows of 36 for 510 x 510; along z 1.10: 2K planes
+// of every run and the last wave); DRAM is at 30%.
 // Measured on 512^3, us per step, warps x rows: K=2 16x3 107, 12x5 106; K=3
 // 12x3 100, 8x5 117, 16x2 125, 12x4 and 8x6 spill (115, 122); K=4 8x4 113.
 #include <math.h>

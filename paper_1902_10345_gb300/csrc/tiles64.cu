@@ -10,7 +10,7 @@
 // that no lane idles, and little is recomputed: the halo is K <= 8 cells, step
 // s of a pass updates the tile and K - s cells around it, and K and the tiling
 // are chosen for the grid (plan_tiles64).  Measured, against a launch per 4
-// steps of the streamed kernel: 256^2 T=100 168 us (1076), 700 x 300 T=100 317
+// steps of the streamed kernel: 256^2 T=100 164 us (1076), 700 x 300 T=100 317
 // (1079), 1000^2 T=50 573 (957), 1400^2 T=30 656 (1225): 90 of about 115
 // GUpdates/s that the pipe allows at the largest, the exchange and the grid's
 // small share per SM at the smallest.
