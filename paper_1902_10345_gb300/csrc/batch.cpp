@@ -353,36 +353,29 @@ static void plan_free(sdfg_batch_plan *p) {
 // - FP64, and below 2^18 points, where a pass is one unit's latency either way;
 // - less than 2^12 points a grid: ms, exact and this, 2000 FP32 grids of 16..64, T=
 //   50..500: 1.65, 2.14;
-// - fewer than 8 steps and 12 M points (BF16 5 M) or more, a short pass or two beside
-//   which the rings' copies count: 512 FP32 grids of 64..2048, T=1 0.24, 0.29; T=4 0.30, 0.31;
-//   16 of 64..600, T=4: 30 us, 26; BF16 32 of 64..2048, T=4: 38, 47;
-// - BF16, 5 M points or more in grids of less than 2^17: 128 grids of 64..512, T=50..
-//   500: 3.0, 3.3 ms; 384 of them 6.2, 6.4, T=7..8 219, 296 us.
+// - 12 M points or more and fewer than 8 steps (BF16 4), a short pass or two beside
+//   which the rings' copies count: 512 grids of 64..2048, us, FP32 T=1 240, 290; T=4 299,
+//   308; T=8 880, 480; BF16 T=1 200, 231; T=4 352, 296; but 16 of 64..600, T=4: 30, 26.
 // Depth 4, for FP32 alone, whose values are not rounded between passes: 12 M points
 // or more in small grids or short runs, where the remainder passes of depth 8 bring
 // more pipe variants in flight: 384 grids of 64..512, T=50..500: depth 8 4.7 ms, 4 3.7;
 // T=13..16 339, 239 us; but 512 of 64..2048, T=50..500: 15.3, 15.8.
 // Segments by the rows that a warp in flight (12 per SM, 112 columns each) has to
 // itself in a pass: few, and the lag from pass to pass counts, many, and the halo
-// rows do; BF16 units move half the bytes and gain from fewer halo rows sooner.
-// Measured at depth 8, ms, T=50..500, grids of 64..2048 if not said, exact and at 64,
-// 128, 256 rows: FP32 32 grids (12 M points) 3.7, 2.3, 2.9, 4.6; 128 (51 M) 9.9, 6.4,
-// 5.7, 6.4; 512 (170 M) 32.3, 21.6, 17.3, 16.1 (384 rows 16.3); 16 of 64..600 (1 M)
-// 2.2, 1.6, 2.5, 4.3; BF16 64 of 64..512 (3 M) 2.5, 2.1, 2.8, 4.4; 32 4.1, 4.1, 3.6,
-// 4.9; 128 10.7, 10.6, 9.2, 9.1 (T=7..8 0.32, -, 0.28, 0.34); 512 34.6, 36, 29.3, 25.6
-// (384 rows 24.0).
+// rows do.  Measured at depth 8, ms, T=50..500, grids of 64..2048 if not said, exact and
+// at 64, 128, 256 rows: FP32 32 grids (12 M points) 3.7, 2.3, 2.9, 4.6; 128 (51 M) 9.9,
+// 6.4, 5.7, 6.4; 512 (170 M) 32.3, 21.6, 17.3, 16.1 (384 rows 16.3); 16 of 64..600 (1 M)
+// 2.2, 1.6, 2.5, 4.3; BF16 16 of 64..600 2.3, 1.7, 2.5, 4.3; 128 of 64..512 (7 M) 3.2, 2.5,
+// 3.0, 4.4; 32 4.1, 2.3, 2.9, 4.8; 128 10.7, 6.2, 5.9, 6.7; 512 34.9, 20.6, 17.9, 16.7.
 static bool untuned_batch(double points, int n, int steps, int dtype, int sm_count, sdfg_config *c) {
     const bool bf16 = dtype == SDFG_BF16;
     const double mean = points / n;
     if (dtype == SDFG_F64 || points < (1 << 18) || mean < (1 << 12)) return false;
-    if (steps < 8 && points >= (bf16 ? 5e6 : 12e6)) return false;
-    if (bf16 && points >= 5e6 && mean < (1 << 17)) return false;
+    if (steps < (bf16 ? 4 : 8) && points >= 12e6) return false;
     const double rows = points / (sm_count * 12.0 * 112.0);
     if (!bf16 && points >= 12e6 && (mean < (1 << 16) || steps < 32)) {
         c->k = 4;
         c->seg_rows = rows < 480 ? 96 : rows < 670 ? 160 : 256;
-    } else if (bf16) {
-        c->seg_rows = rows < 25 ? 64 : rows < 50 ? 96 : rows < 300 ? 128 : rows < 590 ? 256 : 384;
     } else {
         c->seg_rows = rows < 75 ? 64 : rows < 340 ? 128 : 256;
     }

@@ -74,6 +74,7 @@ static __device__ __noinline__ int chain_wait_rows(const int *prog_prev, int bet
 template <int CR>
 struct ChainHook {
     static constexpr bool EDGES = true;
+    static constexpr bool ALL = true;
     static constexpr int TURN = SDFG_CHAIN_TURN;
     static constexpr int ROWS = CR;
     const int *prog_prev;  // counters of pass p-1 (nullptr for pass 0: the input is ready)

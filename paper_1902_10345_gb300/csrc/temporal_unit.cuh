@@ -263,12 +263,14 @@ static_assert(CHUNK_ROWS % SDFG_RING2_TURN == 0, "chunks are whole turns");
 // stream (the chain kernel, skewed.cu).  The whole warp calls ready(c) before
 // chunk c is loaded (false: a bounded wait ran out) and done(c) once chunk c's
 // rows are stored and the warp is synchronised.  EDGES: a unit of the
-// reassociated pipe may hold row 0 or row R-1 (see step2).  The units of the
+// reassociated pipe may hold row 0 or row R-1 (see step2).  ALL: a chunk body
+// without the per-row store test, for BF16 (see run).  The units of the
 // per-pass and persistent kernels need none of it.  TURN: rows per turn of
 // the two-row-ring chunk loop (one unrolled body); the best value differs
 // between the kernels (measured).
 struct NoHook {
     static constexpr bool EDGES = false;
+    static constexpr bool ALL = false;
     static constexpr int TURN = SDFG_RING2_TURN;
     __device__ __forceinline__ bool ready(int) { return true; }
     __device__ __forceinline__ void done(int) {}
@@ -633,10 +635,11 @@ struct UnitPipe {
                 const bool edge = Hook::EDGES && (r0 <= K || (r0 + CR - 2 >= R - 1 && r0 - K <= R - 1));
                 // every output row of the chunk stored (the common case): a
                 // third body without the per-row test, for BF16 chains only
-                // (measured: BF16 +3%; FP32 chains -22% and the persistent
-                // kernel -6%, whose larger hot code it pushes out of the
-                // instruction cache)
-                constexpr bool ALL_BODY = SDFG_RING2_ALL_BODY && sizeof(ST) == 2 && Hook::EDGES;
+                // (measured: BF16 +3%; FP32 chains -22%; the persistent kernel,
+                // whose larger hot code it pushes out of the instruction cache,
+                // -6%, and its scaled BF16 grids, of many depths at once, 512
+                // of 64..2048 16.4 -> 23.2 ms)
+                constexpr bool ALL_BODY = SDFG_RING2_ALL_BODY && sizeof(ST) == 2 && Hook::ALL;
                 const bool all = ALL_BODY && (r0 - K >= sy0) && (r0 + CR - 1 - K < sy1);
                 if (edge)
                     chunk_body2<true, Hook::TURN>(r0, src, out);
