@@ -38,6 +38,12 @@
  *     batch as a whole (see the batch plans), which differ by that tolerance;
  *     among batches that run the same way a grid's result does not depend on
  *     its companions.  Give a configuration for the same bits in any mix.
+ *   - Range of FP32 arithmetic: in the order shown values up to 6.8e37 (3-D
+ *     4.8e37) stay finite and infinities stay infinite.  That holds for every
+ *     call with the defaults but grids on the chain kernel, and units away from
+ *     the ring under a streamed or persistent configuration and in solves, the
+ *     server and exact-order batches: there unscaled sums overflow from
+ *     8.7e32 at k = 8, and an infinity may become NaN.
  *   - BF16 storage: the steps fused into one pass stay in FP32 registers and
  *     values are rounded to BF16 each time a pass writes the grid, so the
  *     result also depends on k; the register tiles round once, at the end.
